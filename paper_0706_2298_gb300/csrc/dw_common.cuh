@@ -55,6 +55,24 @@ template <typename T> DW_HD cplx<T> cmulc(cplx<T> a, cplx<T> b) {
 // i * a
 template <typename T> DW_HD cplx<T> ti(cplx<T> a) { return {-a.im, a.re}; }
 template <typename T> DW_HD T norm2(cplx<T> a) { return a.re * a.re + a.im * a.im; }
+// acc + a b, acc - a b, acc + conj(a) b and the product a b as chains of fused multiply-adds.  Written as
+// operators, acc + a * b costs six instructions (a product's second half is fused with its first, so the
+// sum needs an addition of its own); as a chain it costs four.
+DW_HD float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+DW_HD double fma_(double a, double b, double c) { return fma(a, b, c); }
+template <typename T> DW_HD void rmac(T& acc, T a, T b) { acc = fma_(a, b, acc); }
+template <typename T> DW_HD void cmac(cplx<T>& acc, cplx<T> a, cplx<T> b) {
+  acc.re = fma_(-a.im, b.im, fma_(a.re, b.re, acc.re));
+  acc.im = fma_(a.im, b.re, fma_(a.re, b.im, acc.im));
+}
+template <typename T> DW_HD void cmsub(cplx<T>& acc, cplx<T> a, cplx<T> b) {
+  acc.re = fma_(a.im, b.im, fma_(-a.re, b.re, acc.re));
+  acc.im = fma_(-a.im, b.re, fma_(-a.re, b.im, acc.im));
+}
+template <typename T> DW_HD void cmacc(cplx<T>& acc, cplx<T> a, cplx<T> b) {
+  acc.re = fma_(a.im, b.im, fma_(a.re, b.re, acc.re));
+  acc.im = fma_(-a.im, b.re, fma_(a.re, b.im, acc.im));
+}
 
 // ---------------------------------------------------------------- 16-byte units
 template <typename T> struct Unit;
@@ -104,6 +122,10 @@ DW_D dd operator*(dd a, dd b) {
 }
 DW_D dd& operator+=(dd& a, dd b) { a = a + b; return a; }
 DW_D dd& operator-=(dd& a, dd b) { a = a - b; return a; }
+DW_D void rmac(dd& acc, dd a, dd b) { acc += a * b; }
+DW_D void cmac(cplx<dd>& acc, cplx<dd> a, cplx<dd> b) { acc += a * b; }
+DW_D void cmsub(cplx<dd>& acc, cplx<dd> a, cplx<dd> b) { acc -= a * b; }
+DW_D void cmacc(cplx<dd>& acc, cplx<dd> a, cplx<dd> b) { acc += cmulc(a, b); }
 DW_D double dd_to_double(dd a) { return (double)a.hi + (double)a.lo; }
 DW_D dd __shfl_xor_sync(unsigned mask, dd v, int lane) {
   return {__shfl_xor_sync(mask, v.hi, lane), __shfl_xor_sync(mask, v.lo, lane)};
@@ -206,18 +228,30 @@ DW_D void load_link(const T* __restrict__ links, size_t V, int mu, size_t i, SU3
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     int j1 = (j + 1) % 3, j2 = (j + 2) % 3;
-    U.m[2][j] = conjg(U.m[0][j1] * U.m[1][j2] - U.m[0][j2] * U.m[1][j1]);
+    cplx<T> r2 = U.m[0][j1] * U.m[1][j2];
+    cmsub(r2, U.m[0][j2], U.m[1][j1]);
+    U.m[2][j] = conjg(r2);
   }
 }
 template <typename T>
 DW_D void su3_mul(const SU3<T>& U, const cplx<T>* h, cplx<T>* o) {
 #pragma unroll
-  for (int a = 0; a < 3; ++a) o[a] = U.m[a][0] * h[0] + U.m[a][1] * h[1] + U.m[a][2] * h[2];
+  for (int a = 0; a < 3; ++a) {
+    cplx<T> w = U.m[a][0] * h[0];
+    cmac(w, U.m[a][1], h[1]);
+    cmac(w, U.m[a][2], h[2]);
+    o[a] = w;
+  }
 }
 template <typename T>
 DW_D void su3_dag_mul(const SU3<T>& U, const cplx<T>* h, cplx<T>* o) {
 #pragma unroll
-  for (int a = 0; a < 3; ++a) o[a] = cmulc(U.m[0][a], h[0]) + cmulc(U.m[1][a], h[1]) + cmulc(U.m[2][a], h[2]);
+  for (int a = 0; a < 3; ++a) {
+    cplx<T> w = cmulc(U.m[0][a], h[0]);
+    cmacc(w, U.m[1][a], h[1]);
+    cmacc(w, U.m[2][a], h[2]);
+    o[a] = w;
+  }
 }
 
 // ---------------------------------------------------------------- spin structure
@@ -265,30 +299,39 @@ DW_D void hop_acc(cplx<T>* acc, const cplx<T>* psi, const SU3<T>& U, T sign) {
 }
 
 // ---------------------------------------------------------------- clover
-// y = A x for one chiral block stored in 18 slots (see layout above)
-template <typename T>
+// y = A x for one chiral block stored in 18 slots (see layout above).  LAST: the off-diagonal products are
+// summed first and the diagonal ones, the largest, added last, so that the sums round at the size of the
+// smaller terms (D in FP32: 6e-8 instead of 9e-8 from FP64, at the same speed).  The Schwarz kernels, at
+// their register limit, add to the diagonal products instead (the other order spills, 1.44 -> 2.40 ms).
+template <bool LAST = false, typename T>
 DW_D void herm6_mul(const cplx<T>* s, const cplx<T>* x, cplx<T>* y) {
   const T d[6] = {s[0].re, s[0].im, s[1].re, s[1].im, s[2].re, s[2].im};
+  if (!LAST) {
 #pragma unroll
-  for (int i = 0; i < 6; ++i) y[i] = d[i] * x[i];
+    for (int i = 0; i < 6; ++i) y[i] = d[i] * x[i];
+  }
   int k = 3;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
 #pragma unroll
     for (int j = i + 1; j < 6; ++j) {
-      y[i] += s[k] * x[j];
-      y[j] += cmulc(s[k], x[i]);
+      if (LAST && i == 0 && j == 1) y[0] = s[k] * x[j]; else cmac(y[i], s[k], x[j]);
+      if (LAST && i == 0) y[j] = cmulc(s[k], x[0]); else cmacc(y[j], s[k], x[i]);
       ++k;
     }
   }
+  if (LAST) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) { rmac(y[i].re, d[i], x[i].re); rmac(y[i].im, d[i], x[i].im); }
+  }
 }
-template <typename T>
+template <bool LAST = false, typename T>
 DW_D void clover_apply(const T* __restrict__ clov, size_t V, size_t i, const cplx<T>* x, cplx<T>* y) {
   cplx<T> s[18];
   load_site<T, 18>(clov, V, i, s);
-  herm6_mul(s, x, y);
+  herm6_mul<LAST>(s, x, y);
   load_site<T, 18>(clov + 36 * V, V, i, s);
-  herm6_mul(s, x + 6, y + 6);
+  herm6_mul<LAST>(s, x + 6, y + 6);
 }
 
 // ---------------------------------------------------------------- contexts
@@ -325,6 +368,7 @@ struct WsArena {
 struct dw_ctx {
   dw_params p;
   int device = -1;             // CUDA device the context's memory lives on (current device at dw_create)
+  int sms = 0;                 // its multiprocessors
   uint64_t gauge_hash = 0;     // FNV-1a hash of the links given to dw_create (identifies the gauge field)
   Geom g;                      // device pointers filled in
   long long V;
@@ -353,8 +397,8 @@ struct dw_ctx {
   double* d_red = nullptr;                // reduction scratch
   unsigned* d_count = nullptr;
   double* h_red = nullptr;                // pinned host mirror
-  WsArena ws_solve[4];                    // solver workspaces: [0] GCR, [1] batched GCR, [2] CGNR and
-                                          // BiCGstab, [3] low-mode subspace iteration
+  WsArena ws_solve[5];                    // solver workspaces: [0] GCR, [1] batched GCR, [2] CGNR and
+                                          // BiCGstab, [3] low-mode subspace iteration, [4] network training
 };
 
 // DW_OK when the calling thread's current device is the context's device; otherwise DW_EINVAL

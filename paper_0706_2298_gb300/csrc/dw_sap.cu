@@ -186,8 +186,8 @@ __global__ void __launch_bounds__(SHV) sap_block_kernel(Geom g, const T* __restr
     if (pp > 0) alpha = {(T)(pr / pp), (T)(pi / pp)};
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      x[k] += alpha * v[k];
-      v[k] -= alpha * w[k];
+      cmac(x[k], alpha, v[k]);
+      cmsub(v[k], alpha, w[k]);
       s_r[k * SHV + h] = v[k];
     }
     __syncthreads();                                        // s_red reused, s_r complete
@@ -226,262 +226,531 @@ __global__ void __launch_bounds__(SHV) sap_block_kernel(Geom g, const T* __restr
 }
 
 // ============================================================================ staged FP32 kernel
-// Same algorithm as sap_block_kernel, organised for throughput:
-//  * the block's links are staged once into shared memory as full 3x3 matrices;
-//  * 2*SHV threads: lanes 2h and 2h+1 (q = 0, 1) share the site pair h.  In the
-//    hopping sums each thread projects onto spin q only: it loads half of each
-//    neighbour spinor and does one SU(3) product per hop.  Two lane-pair shuffles
-//    then regroup the sum by chirality: thread q owns chiral block q
-//    (spins 2q, 2q+1 = components 6q..6q+5) of both sites, applies that 6x6 clover
-//    block and keeps its share of the MR vectors.
-// acc layout of a thread's hop share: [0..2] upper spin q, [3..5] lower spin 2+q, [6..8] lower spin 3-q
-
-// z * (sgn) or z * (i sgn)
-template <bool IMAG>
-DW_D cplx<float> unit_mul(cplx<float> z, float sgn) {
-  if (IMAG) return {-sgn * z.im, sgn * z.re};
-  return {sgn * z.re, sgn * z.im};
-}
-
-template <int MU>
-DW_D void half_hop_dir(const cplx<float>* __restrict__ sU, const cplx<float>* __restrict__ sm, int SHV, int lown,
-                       int lnb_base, uint16_t ef, uint16_t eb, int q, cplx<float>* acc) {
-  constexpr int NSITE_MUL = 2;
-  (void)NSITE_MUL;
-  const int NS = 2 * SHV;
-  // e_mu psi_lo coefficient for spin q and the spin it takes from the lower half
-  constexpr bool IM = (MU == 1 || MU == 3);
-  const float sg = (MU == 0 || MU == 1) ? -1.f : (q ? 1.f : -1.f);
-  const int lo = (MU == 0 || MU == 3) ? 2 + q : 3 - q;
-  const int slot = (MU == 0 || MU == 3) ? 3 : 6;       // accumulator of the lower spin touched
-  if (!(ef >> 15)) {                                   // forward: (1 - gamma) U(x) psi(x+mu)
-    const int hn = ef & 0x7fff;
-    cplx<float> hv[3], w[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) hv[c] = sm[(3 * q + c) * SHV + hn] - unit_mul<IM>(sm[(3 * lo + c) * SHV + hn], sg);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const cplx<float>* u = sU + (MU * 9 + 3 * a) * NS + lown;
-      w[a] = u[0] * hv[0] + u[NS] * hv[1] + u[2 * NS] * hv[2];
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      acc[c] += w[c];
-      acc[slot + c] -= unit_mul<IM>(w[c], IM ? -sg : sg);   // S = -1, coefficient conj(e)
-    }
-  }
-  if (!(eb >> 15)) {                                   // backward: (1 + gamma) U(x-mu)^+ psi(x-mu)
-    const int hn = eb & 0x7fff;
-    const int ln = lnb_base + hn;
-    cplx<float> hv[3], w[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) hv[c] = sm[(3 * q + c) * SHV + hn] + unit_mul<IM>(sm[(3 * lo + c) * SHV + hn], sg);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const cplx<float>* u = sU + (MU * 9 + a) * NS + ln;
-      w[a] = cmulc(u[0], hv[0]) + cmulc(u[3 * NS], hv[1]) + cmulc(u[6 * NS], hv[2]);
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      acc[c] += w[c];
-      acc[slot + c] += unit_mul<IM>(w[c], IM ? -sg : sg);
-    }
-  }
-}
-
-// hop share at a site -> this thread's chiral block (6 complex) of the full hopping sum
-DW_D void staged_hops(const cplx<float>* sU, const cplx<float>* sm, int SHV, int p, int h, int q,
-                      const uint16_t* nbe, cplx<float>* out6) {
-  cplx<float> acc[9];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) acc[k] = {0.f, 0.f};
-  const int lown = p * SHV + h, lnb = (1 - p) * SHV;
-  half_hop_dir<0>(sU, sm, SHV, lown, lnb, nbe[0], nbe[1], q, acc);
-  half_hop_dir<1>(sU, sm, SHV, lown, lnb, nbe[2], nbe[3], q, acc);
-  half_hop_dir<2>(sU, sm, SHV, lown, lnb, nbe[4], nbe[5], q, acc);
-  half_hop_dir<3>(sU, sm, SHV, lown, lnb, nbe[6], nbe[7], q, acc);
-  // lower spin 2+q: own slot 3 + partner's slot 6 (its 3-q' = 2+q)
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    float re = __shfl_xor_sync(0xffffffffu, acc[6 + c].re, 1);
-    float im = __shfl_xor_sync(0xffffffffu, acc[6 + c].im, 1);
-    acc[3 + c] += cplx<float>{re, im};
-  }
-  // thread q holds spins q (upper) and 2+q (lower); chiral block q needs spins 2q, 2q+1:
-  // q = 0 keeps spin 0 and receives spin 1; q = 1 keeps spin 3 and receives spin 2
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    cplx<float> send = q ? acc[c] : acc[3 + c];          // q=1 sends spin 1, q=0 sends spin 2
-    float re = __shfl_xor_sync(0xffffffffu, send.re, 1);
-    float im = __shfl_xor_sync(0xffffffffu, send.im, 1);
-    if (q == 0) { out6[c] = acc[c]; out6[3 + c] = {re, im}; }
-    else        { out6[c] = {re, im}; out6[3 + c] = acc[3 + c]; }
-  }
-}
-
-DW_D void clover_block(const float* __restrict__ cl, size_t V, long long i, int q, const cplx<float>* x,
-                       cplx<float>* y) {
-  cplx<float> s[18];
-  load_site<float, 18>(cl + (size_t)36 * V * q, V, i, s);
-  herm6_mul(s, x, y);
-}
-
+// Same algorithm as sap_block_kernel, one thread per site of the block (thread t = site t: the even
+// sites first, then the odd ones).  Every link product is done by the thread that owns the link:
+//   * forward term of a hop: the destination x reads psi(x + mu) from shared memory and multiplies it
+//     by its own U_mu(x);
+//   * backward term: the source y forms U_mu(y)^+ (1 + gamma_mu) psi(y) from its own registers and
+//     hands the half-spinor to y + mu through shared memory.
+// So both parities work in each hop, and a link and a clover block are read by one thread only: they
+// need not be in shared memory.  Blocks of 128 and 256 sites keep the links (72 reals per thread) and
+// one chiral block of A_ee / A_oo^{-1} (36 reals) in tensor memory, used as a second register file
+// (tcgen05.st / tcgen05.ld 32x32b: a thread's columns of its lane), the other chiral block, the vector,
+// the half-spinors and x_e / b_o in shared memory: a block solve reads nothing from L2 between its first
+// and last access.  Smaller blocks keep the links in shared memory and read the clover term from L2.
+// While the odd sites apply A_oo^{-1}, the even ones apply A_ee.
+// Bound: instruction issue and latency (16 warps per SM at 128 registers and 98 KB, issue slots 57% busy);
+// the rest is the two parities waiting for each other and tensor-memory loads.  48x24^3 on 4^4 blocks, 4
+// cycles of 4 steps: 1.44 ms (22 TFLOP/s); links in shared memory and the whole clover term in tensor
+// memory 1.60 ms; pulling both hop terms from shared memory with one thread per (site pair, spin) 1.78 ms.
 template <int SHV>
-__global__ void __launch_bounds__(2 * SHV, 2) sap_staged_kernel(Geom g, const float* __restrict__ links,
-                                                                const float* __restrict__ clov,
-                                                                const float* __restrict__ clovinv,
-                                                                const int* __restrict__ blocks, const float* rsrc0,
-                                                                float* rdst0, const float* dprev0, float* dout0,
-                                                                float* xi0, int first, int nmr, int nrhs,
-                                                                size_t fstride) {
-  constexpr int NT = 2 * SHV, NS = 2 * SHV, NW = NT / 32;
+struct SapCfg {
+  static constexpr int NS = 2 * SHV;
+  static constexpr bool TM = SHV >= 64;
+  [[maybe_unused]] static constexpr int TCOLS = SHV >= 128 ? 256 : 128;       // columns of a CTA: 128 per warp of a lane quarter
+  static constexpr int FIXED = TM ? NS * 144 : NS * 288;      // clover block 1, or the links
+  static constexpr size_t bytes = (size_t)FIXED + (size_t)SHV * (12 + 6 + 12) * 16;
+};
+
+DW_D void tm_st16(uint32_t a, const float* v) {
+  const uint32_t* r = reinterpret_cast<const uint32_t*>(v);
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+      ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+      "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
+DW_D void tm_st2(uint32_t a, const float* v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};" ::"r"(a), "r"(__float_as_uint(v[0])),
+               "r"(__float_as_uint(v[1])) : "memory");
+}
+DW_D void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// 18 consecutive columns (the wait is part of the statement: the registers are valid after it)
+DW_D void tm_ld18(uint32_t a, float* v) {
+  uint32_t r[18];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%18];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%16,%17}, [%19];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17])
+      : "r"(a), "r"(a + 16) : "memory");
+#pragma unroll
+  for (int k = 0; k < 18; ++k) v[k] = __uint_as_float(r[k]);
+}
+
+// CTA barriers of a subset: wait for, or only announce, the arrival of n threads at barrier id
+DW_D void bar_wait(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+DW_D void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+// the block's data as thread t sees it
+template <int SHV>
+struct SapBlock {
+  using Cfg = SapCfg<SHV>;
+  static constexpr int NS = 2 * SHV;
+  float4* fix4;     // TM: clover block 1, [9 units][NS]; else the links' complex 0..7, [4 mu][4 units][NS]
+  float2* fix2;     // else: complex 8 of the links, [4 mu][NS]
+  float4* half;     // [4 mu][3 units][SHV]  half-spinors of the backward terms, at the source's index
+  float4* vec;      // [6 units][SHV]        r_e, t_o or x_e
+  float4* xb;       // [6 units][NS]         x_e on the even sites, b_o on the odd ones
+  uint32_t tm;      // this thread's tensor-memory address
+  const float* cl;  // else: A_oo^{-1} (odd t) or A_ee (even t) in global memory
+  int t;
+
+  DW_D void set(unsigned char* p, int thread) {
+    t = thread;
+    fix4 = reinterpret_cast<float4*>(p);
+    fix2 = reinterpret_cast<float2*>(p + (size_t)NS * 256);
+    half = reinterpret_cast<float4*>(p + Cfg::FIXED);
+    vec = half + 12 * SHV;
+    xb = vec + 6 * SHV;
+  }
+  DW_D void stage(const float* __restrict__ links, const float* __restrict__ clover, size_t V, long long i) {
+    cl = clover;
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+      SU3<float> U;
+      load_link(links, V, mu, i, U);
+      if constexpr (Cfg::TM) {
+        tm_st16(tm + mu * 18, &U.m[0][0].re);
+        tm_st2(tm + mu * 18 + 16, &U.m[2][2].re);
+      } else {
+        const cplx<float>* m = &U.m[0][0];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) fix4[(mu * 4 + k) * NS + t] = pack_unit(m + 2 * k);
+        fix2[mu * NS + t] = make_float2(m[8].re, m[8].im);
+      }
+    }
+    if constexpr (Cfg::TM) {
+      cplx<float> s[18];
+      load_site<float, 18>(clover, V, i, s);
+      tm_st16(tm + 72, &s[0].re);
+      tm_st2(tm + 88, &s[8].re);
+      tm_st16(tm + 90, &s[9].re);
+      tm_st2(tm + 106, &s[17].re);
+      const float4* q = reinterpret_cast<const float4*>(clover + 36 * V);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) fix4[k * NS + t] = __ldg(q + (size_t)k * V + i);
+      tm_wait_st();
+    }
+  }
+  DW_D void link(int mu, SU3<float>& U) const {      // whole warps only (tensor memory)
+    cplx<float>* m = &U.m[0][0];
+    if constexpr (Cfg::TM) {
+      tm_ld18(tm + mu * 18, &m[0].re);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) unpack_unit(fix4[(mu * 4 + k) * NS + t], m + 2 * k);
+      const float2 l = fix2[mu * NS + t];
+      m[8] = {l.x, l.y};
+    }
+  }
+  // y = A_oo^{-1} x (odd) or A_ee x (even)
+  DW_D void clover(size_t V, long long i, const cplx<float>* x, cplx<float>* y) const {
+    cplx<float> s[18];
+    if constexpr (Cfg::TM) {
+      tm_ld18(tm + 72, &s[0].re);
+      tm_ld18(tm + 90, &s[9].re);
+      herm6_mul(s, x, y);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) unpack_unit(fix4[k * NS + t], s + 2 * k);
+      herm6_mul(s, x + 6, y + 6);
+    } else {
+      clover_apply(cl, V, i, x, y);
+    }
+  }
+  DW_D void put(float4* a, int stride, int at, const cplx<float>* f) const {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) a[k * stride + at] = pack_unit(f + 2 * k);
+  }
+  DW_D void get(const float4* a, int stride, int at, cplx<float>* f) const {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) unpack_unit(a[k * stride + at], f + 2 * k);
+  }
+};
+
+// the eight neighbour-table entries of a site (direction 2 mu forward, 2 mu + 1 backward)
+struct SapNb {
+  uint32_t w[4];
+  DW_D bool in(int d) const { return !((w[d >> 1] >> ((d & 1) * 16 + 15)) & 1u); }
+  DW_D int at(int d) const { return (int)((w[d >> 1] >> ((d & 1) * 16)) & 0x7fffu); }
+};
+
+// half-spinor w = W (1 + S gamma_mu) psi, W = U or U^+
+template <int MU, int S, bool DAG>
+DW_D void half_spinor(const cplx<float>* psi, const SU3<float>& U, cplx<float>* w) {
+  cplx<float> hs[2][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    cplx<float> v0, v1;
+    e_mul<MU>(psi[6 + c], psi[9 + c], v0, v1);
+    if (S > 0) { hs[0][c] = psi[c] + v0; hs[1][c] = psi[3 + c] + v1; }
+    else       { hs[0][c] = psi[c] - v0; hs[1][c] = psi[3 + c] - v1; }
+  }
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    if (DAG) su3_dag_mul(U, hs[a], w + 3 * a); else su3_mul(U, hs[a], w + 3 * a);
+  }
+}
+// acc += the spinor [w ; S e_mu^+ w] of a half-spinor
+template <int MU, int S>
+DW_D void add_half(const cplx<float>* w, cplx<float>* acc) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    cplx<float> l0, l1;
+    edag_mul<MU>(w[c], w[3 + c], l0, l1);
+    acc[c] += w[c];
+    acc[3 + c] += w[3 + c];
+    if (S > 0) { acc[6 + c] += l0; acc[9 + c] += l1; }
+    else       { acc[6 + c] -= l0; acc[9 + c] -= l1; }
+  }
+}
+
+// acc += (1 - gamma_mu) U_mu(x) psi(x + mu), psi in the shared vector
+template <int MU, int SHV>
+DW_D void sap_forward(const SapBlock<SHV>& sb, const SapNb& nb, cplx<float>* acc) {
+  SU3<float> U;
+  sb.link(MU, U);
+  if (nb.in(2 * MU)) {
+    cplx<float> p[12], w[6];
+    sb.get(sb.vec, SHV, nb.at(2 * MU), p);
+    half_spinor<MU, -1, false>(p, U, w);
+    add_half<MU, -1>(w, acc);
+  }
+}
+// half-spinors U_mu(y)^+ (1 + gamma_mu) psi(y) of the owner's spinor
+template <int MU, int SHV>
+DW_D void sap_push(const SapBlock<SHV>& sb, const SapNb& nb, int h, const cplx<float>* psi) {
+  SU3<float> U;
+  sb.link(MU, U);
+  if (nb.in(2 * MU)) {
+    cplx<float> w[6];
+    half_spinor<MU, +1, true>(psi, U, w);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) sb.half[(MU * 3 + k) * SHV + h] = pack_unit(w + 2 * k);
+  }
+}
+// acc += the backward term of direction mu, from the half-spinor of x - mu
+template <int MU, int SHV>
+DW_D void sap_gather(const SapBlock<SHV>& sb, const SapNb& nb, cplx<float>* acc) {
+  if (nb.in(2 * MU + 1)) {
+    const int hn = nb.at(2 * MU + 1);
+    cplx<float> w[6];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) unpack_unit(sb.half[(MU * 3 + k) * SHV + hn], w + 2 * k);
+    add_half<MU, +1>(w, acc);
+  }
+}
+
+// Halo of a block: the hops of the neighbouring blocks' last correction f into the block's boundary
+// sites.  One thread per (face, site of the face) forms the half-spinor, so that no lane idles on
+// interior sites; the boundary sites then collect them from shared memory ([3 units][items], in the
+// space of half, vec and xb, which is large enough for every block of 2 SHV sites).
+struct SapFaces {
+  uint32_t pos, wid;               // bytes: bit position and width of coordinate mu in the local index
+  int off[9];                      // first item of each face (constant subscripts only)
+  DW_D explicit SapFaces(const Geom& g) : pos(0), wid(0) {
+    int at = 0;
+#pragma unroll
+    for (int mu = 3; mu >= 0; --mu) {
+      const int w = 31 - __clz(g.sb[mu]);
+      pos |= (uint32_t)at << (8 * mu);
+      wid |= (uint32_t)w << (8 * mu);
+      at += w;
+    }
+    off[0] = 0;
+#pragma unroll
+    for (int d = 0; d < 8; ++d) off[d + 1] = off[d] + (g.svol >> width(d >> 1));
+  }
+  DW_D int shift(int mu) const { return (int)((pos >> (8 * mu)) & 255u); }
+  DW_D int width(int mu) const { return (int)((wid >> (8 * mu)) & 255u); }
+  // local lexicographic index of face site j of direction d (forward: the last coordinate, backward: 0)
+  DW_D int lex(int d, int j) const {
+    const int s = shift(d >> 1), w = width(d >> 1), lo = j & ((1 << s) - 1);
+    return ((j - lo) << w) | (((d & 1) ? 0 : (1 << w) - 1) << s) | lo;
+  }
+  DW_D int face(int d, int lx) const {
+    const int s = shift(d >> 1), lo = lx & ((1 << s) - 1);
+    return ((lx >> (s + width(d >> 1))) << s) | lo;
+  }
+  DW_D int parity(int lx) const { return ((lx >> shift(0)) ^ (lx >> shift(1)) ^ (lx >> shift(2)) ^ lx) & 1; }
+};
+
+template <int D>
+DW_D void halo_item(const Geom& g, const SiteRef& s, long long i, const float* __restrict__ links, const float* f,
+                    cplx<float>* w) {
+  bool cr;
+  const long long j = neighbour(g, s, D, &cr);
+  SU3<float> U;
+  cplx<float> p[12];
+  load_link(links, (size_t)g.V, D >> 1, (D & 1) ? j : i, U);
+  load_site_rw<float, 12>(f, (size_t)g.V, j, p);
+  half_spinor<(D >> 1), (D & 1) ? +1 : -1, (D & 1) != 0>(p, U, w);
+}
+
+template <int D, int SHV>
+DW_D void halo_gather(const SapFaces& fc, const float4* buf, const SapNb& nb, int lx, bool wrap, cplx<float>* acc) {
+  if (nb.in(D)) return;
+  const int at = fc.off[D] + fc.face(D, lx), n = fc.off[8];
+  cplx<float> w[6];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) unpack_unit(buf[k * n + at], w + 2 * k);
+  if (wrap) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) w[k] = -w[k];
+  }
+  add_half<(D >> 1), (D & 1) ? +1 : -1>(w, acc);
+}
+
+// b += 1/2 hops of f across the block boundary (r - D delta on the boundary); all threads, with barriers
+template <int SHV>
+DW_D void sap_halo(const Geom& g, const SapBlock<SHV>& sb, const SapNb& nb, int b, const float* __restrict__ links,
+                   const float* f, cplx<float>* v) {
+  const SapFaces fc(g);
+  float4* buf = sb.half;
+  const int n = fc.off[8], t = sb.t;
+  for (int it = t; it < n; it += 2 * SHV) {
+    int d = 0, o = 0;
+#pragma unroll
+    for (int q = 1; q < 8; ++q)
+      if (it >= fc.off[q]) { d = q; o = fc.off[q]; }
+    const int lx = fc.lex(d, it - o);
+    const SiteRef s = {b, fc.parity(lx), lx >> 1};
+    const long long i = site_index(g, b, s.p, s.h);
+    cplx<float> w[6];
+    switch (d) {
+      case 0: halo_item<0>(g, s, i, links, f, w); break;
+      case 1: halo_item<1>(g, s, i, links, f, w); break;
+      case 2: halo_item<2>(g, s, i, links, f, w); break;
+      case 3: halo_item<3>(g, s, i, links, f, w); break;
+      case 4: halo_item<4>(g, s, i, links, f, w); break;
+      case 5: halo_item<5>(g, s, i, links, f, w); break;
+      case 6: halo_item<6>(g, s, i, links, f, w); break;
+      default: halo_item<7>(g, s, i, links, f, w); break;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) buf[k * n + it] = pack_unit(w + 2 * k);
+  }
+  __syncthreads();
+  const int p = t >= SHV ? 1 : 0, h = t - p * SHV;
+  int lx = 2 * h;
+  lx |= fc.parity(lx) ^ p;
+  const SiteRef s = {b, p, h};
+  cplx<float> acc[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = {0.f, 0.f};
+  halo_gather<0, SHV>(fc, buf, nb, lx, time_wrap(g, s, 0), acc);
+  halo_gather<1, SHV>(fc, buf, nb, lx, time_wrap(g, s, 1), acc);
+  halo_gather<2, SHV>(fc, buf, nb, lx, false, acc);
+  halo_gather<3, SHV>(fc, buf, nb, lx, false, acc);
+  halo_gather<4, SHV>(fc, buf, nb, lx, false, acc);
+  halo_gather<5, SHV>(fc, buf, nb, lx, false, acc);
+  halo_gather<6, SHV>(fc, buf, nb, lx, false, acc);
+  halo_gather<7, SHV>(fc, buf, nb, lx, false, acc);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) v[k] += 0.5f * acc[k];
+  __syncthreads();
+}
+
+// right-hand sides rpc blockIdx.y .. of the blocks of one colour
+template <int SHV>
+__global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
+    Geom g, const float* __restrict__ links, const float* __restrict__ clov, const float* __restrict__ clovinv,
+    const int* __restrict__ blocks, const float* rsrc0, float* rdst0, const float* dprev0, float* dout0, float* xi0,
+    int first, int nmr, int nrhs, int rpc, size_t fstride) {
+  using Cfg = SapCfg<SHV>;
+  constexpr int NW = SHV > 32 ? SHV / 32 : 1, NS = 2 * SHV;     // NW: warps of even sites
   extern __shared__ __align__(16) unsigned char sap_smem[];
-  cplx<float>* sU = reinterpret_cast<cplx<float>*>(sap_smem);   // [4][9][NS]
-  cplx<float>* s_r = sU + 36 * NS;                                // [12][SHV] even field
-  cplx<float>* s_t = s_r + 12 * SHV;                              // [12][SHV] odd field, later x_e
-  cplx<float>* s_b = s_t + 12 * SHV;                              // [12][SHV] b_o
   __shared__ float s_red[3][NW];
+  __shared__ uint32_t s_tm;
   const size_t V = g.V;
-  const int t = threadIdx.x, h = t >> 1, q = t & 1;
+  const int t = threadIdx.x, p = t >= SHV ? 1 : 0, h = t - p * SHV;
   const int b = blocks[blockIdx.x];
-  const long long base = (long long)b << g.lsvol;
-  const long long ie = base + h, io = base + SHV + h;
-  // ---- stage the block's links (full matrices)
-  for (int idx = t; idx < 4 * NS; idx += NT) {
-    const int mu = idx / NS, l = idx - mu * NS;
-    SU3<float> U;
-    load_link(links, V, mu, base + l, U);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) sU[(mu * 9 + 3 * a + c) * NS + l] = U.m[a][c];
+  const long long i = ((long long)b << g.lsvol) + t;
+  SapBlock<SHV> sb;
+  sb.set(sap_smem, t);
+  if constexpr (Cfg::TM) {
+    if (t < 32) {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tm)),
+                   "r"((uint32_t)Cfg::TCOLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const int w = t >> 5;        // warp w reads lanes 32 (w mod 4) .. and the columns of its group of four warps
+    sb.tm = s_tm + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(w >> 2) * 128u;
   }
-  uint16_t nbe_e[8], nbe_o[8];
-#pragma unroll
-  for (int d = 0; d < 8; ++d) {
-    nbe_e[d] = __ldg(g.nbtab + (h << 3) + d);
-    nbe_o[d] = __ldg(g.nbtab + ((SHV + h) << 3) + d);
-  }
-  // the staged links serve every right-hand side of the batch
-  for (int rhs = 0; rhs < nrhs; ++rhs) {
-  const size_t fo = (size_t)rhs * fstride;
-  const float* rsrc = rsrc0 + fo;
-  float* rdst = rdst0 ? rdst0 + fo : nullptr;
-  const float* dprev = dprev0 ? dprev0 + fo : nullptr;
-  float* dout = dout0 ? dout0 + fo : nullptr;
-  float* xi = xi0 + fo;
-  // ---- residual with halo correction: q = 0 takes the even site, q = 1 the odd site
+  sb.stage(links, p ? clovinv : clov, V, i);
+  SapNb nb;
   {
-    cplx<float> v[12];
-    const long long i = q ? io : ie;
-    load_site_rw<float, 12>(rsrc, V, i, v);
-    if (dprev) {
-      SiteRef sr = {b, q, h};
-      halo_add(g, sr, i, q ? nbe_o : nbe_e, links, dprev, v);
-    }
-    cplx<float>* dst = q ? s_b : s_r;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) dst[k * SHV + h] = v[k];
+    const uint4 e = __ldg(reinterpret_cast<const uint4*>(g.nbtab) + t);
+    nb.w[0] = e.x; nb.w[1] = e.y; nb.w[2] = e.z; nb.w[3] = e.w;
   }
-  __syncthreads();
-  cplx<float> v6[6], w6[6], h6[6], x6[6];
-  // t_o = A_oo^{-1} b_o  (chiral block q)
+  const int rhs1 = min(nrhs, (int)(blockIdx.y + 1) * rpc);
+  for (int rhs = blockIdx.y * rpc; rhs < rhs1; ++rhs) {
+    const size_t fo = (size_t)rhs * fstride;
+    // f: the field this thread's site contributes to hops (t_o; r^_e, finally x_e); a: hop sums
+    cplx<float> f[12], a[12];
+    load_site_rw<float, 12>(rsrc0 + fo, V, i, f);
+    if (dprev0) sap_halo<SHV>(g, sb, nb, b, links, dprev0 + fo, f);
 #pragma unroll
-  for (int j = 0; j < 6; ++j) v6[j] = s_b[(6 * q + j) * SHV + h];
-  clover_block(clovinv, V, io, q, v6, w6);
+    for (int k = 0; k < 12; ++k) a[k] = {0.f, 0.f};
+    if (p) {                                  // b_o aside, t_o = A_oo^{-1} b_o
+      sb.put(sb.xb, NS, t, f);
+      sb.clover(V, i, f, a);
 #pragma unroll
-  for (int j = 0; j < 6; ++j) s_t[(6 * q + j) * SHV + h] = w6[j];
-  __syncthreads();
-  // r^_e = b_e - D_eo t_o = b_e + 1/2 hops
-  staged_hops(sU, s_t, SHV, 0, h, q, nbe_e, h6);
-#pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    cplx<float> r = s_r[(6 * q + j) * SHV + h] + 0.5f * h6[j];
-    s_r[(6 * q + j) * SHV + h] = r;
-    x6[j] = {0.f, 0.f};
-  }
-  __syncthreads();
-  for (int it = 0; it < nmr; ++it) {
-    // t_o = A_oo^{-1} D_oe r^_e
-    staged_hops(sU, s_r, SHV, 1, h, q, nbe_o, h6);
-#pragma unroll
-    for (int j = 0; j < 6; ++j) v6[j] = -0.5f * h6[j];
-    clover_block(clovinv, V, io, q, v6, w6);
-#pragma unroll
-    for (int j = 0; j < 6; ++j) s_t[(6 * q + j) * SHV + h] = w6[j];
-    __syncthreads();
-    // p = A_ee r^ - D_eo t_o
-#pragma unroll
-    for (int j = 0; j < 6; ++j) v6[j] = s_r[(6 * q + j) * SHV + h];
-    clover_block(clov, V, ie, q, v6, w6);
-    staged_hops(sU, s_t, SHV, 0, h, q, nbe_e, h6);
-    float pr = 0.f, pi = 0.f, pp = 0.f;
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      w6[j] += 0.5f * h6[j];
-      pr += w6[j].re * v6[j].re + w6[j].im * v6[j].im;
-      pi += w6[j].re * v6[j].im - w6[j].im * v6[j].re;
-      pp += w6[j].re * w6[j].re + w6[j].im * w6[j].im;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      pr += __shfl_xor_sync(0xffffffffu, pr, o);
-      pi += __shfl_xor_sync(0xffffffffu, pi, o);
-      pp += __shfl_xor_sync(0xffffffffu, pp, o);
-    }
-    if ((t & 31) == 0) { s_red[0][t >> 5] = pr; s_red[1][t >> 5] = pi; s_red[2][t >> 5] = pp; }
-    __syncthreads();
-    pr = 0.f; pi = 0.f; pp = 0.f;
-#pragma unroll
-    for (int j = 0; j < NW; ++j) { pr += s_red[0][j]; pi += s_red[1][j]; pp += s_red[2][j]; }
-    cplx<float> alpha = {0.f, 0.f};
-    if (pp > 0.f) alpha = {pr / pp, pi / pp};
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      x6[j] += alpha * v6[j];
-      v6[j] -= alpha * w6[j];
-      s_r[(6 * q + j) * SHV + h] = v6[j];
+      for (int k = 0; k < 12; ++k) { f[k] = a[k]; a[k] = {0.f, 0.f}; }
+      sb.put(sb.vec, SHV, h, f);
+    } else {
+      sb.put(sb.xb, NS, t, a);                // x_e = 0
     }
     __syncthreads();
-  }
-  // x_o = A_oo^{-1}(b_o - D_oe x_e)
+    // half steps: s even: r^_e (s = 0) or D^ r^_e from t_o; s odd: t_o from r^_e (last: x_o from x_e)
+    const int last = 2 * nmr + 1;
+    for (int s = 0; s <= last; ++s) {
+      const int dst = s & 1;
+      if (p == dst) {
+        sap_forward<0>(sb, nb, a);
+        sap_forward<1>(sb, nb, a);
+        sap_forward<2>(sb, nb, a);
+        sap_forward<3>(sb, nb, a);
+      } else {
+        sap_push<0>(sb, nb, h, f);
+        sap_push<1>(sb, nb, h, f);
+        sap_push<2>(sb, nb, h, f);
+        sap_push<3>(sb, nb, h, f);
+      }
+      // the half-spinors are complete; their writers need not wait
+      if (SHV < 32) __syncthreads();
+      else if (p == dst) bar_wait(1, NS);
+      else bar_arrive(1, NS);
+      if (p == dst) {
+        sap_gather<0>(sb, nb, a);
+        sap_gather<1>(sb, nb, a);
+        sap_gather<2>(sb, nb, a);
+        sap_gather<3>(sb, nb, a);
+      }
+      if (dst) {
+        // odd: t_o = -1/2 A_oo^{-1} hops, or at the end x_o = A_oo^{-1}(b_o + 1/2 hops);
+        // even: 2 A_ee r^ (doubled: the hops added to it are halved below)
+        cplx<float> y[12];
+        if (p) {
+          if (s == last) sb.get(sb.xb, NS, t, f);
 #pragma unroll
-  for (int j = 0; j < 6; ++j) s_t[(6 * q + j) * SHV + h] = x6[j];
-  __syncthreads();
-  staged_hops(sU, s_t, SHV, 1, h, q, nbe_o, h6);
+          for (int k = 0; k < 12; ++k) f[k] = s == last ? f[k] + 0.5f * a[k] : -0.5f * a[k];
+        }
+        if (p || s < last) {
+          sb.clover(V, i, f, y);
 #pragma unroll
-  for (int j = 0; j < 6; ++j) v6[j] = s_b[(6 * q + j) * SHV + h] + 0.5f * h6[j];
-  clover_block(clovinv, V, io, q, v6, w6);   // w6 = x_o (block q)
-  // ---- outputs: this thread's three float4 units (components 6q..6q+5) of each site
-  float4* dv = reinterpret_cast<float4*>(dout);
-  float4* rv = reinterpret_cast<float4*>(rdst);
-  float4* xv = reinterpret_cast<float4*>(xi);
+          for (int k = 0; k < 12; ++k) {
+            if (p) { f[k] = y[k]; a[k] = {0.f, 0.f}; }
+            else a[k] = 2.f * y[k];
+          }
+        }
+        if (s == last) break;
+        if (p) sb.put(sb.vec, SHV, h, f);
+      } else {
+        if (s == 0) {                         // r^_e = b_e - D_eo t_o = b_e + 1/2 hops
+          if (!p) {
 #pragma unroll
-  for (int u = 0; u < 3; ++u) {
-    const size_t pe = (size_t)(3 * q + u) * V + ie, po = (size_t)(3 * q + u) * V + io;
-    float4 xe = pack_unit(x6 + 2 * u), xo = pack_unit(w6 + 2 * u);
-    if (dout) { dv[pe] = xe; dv[po] = xo; }
-    if (rdst) {
-      cplx<float> r2[2] = {s_r[(6 * q + 2 * u) * SHV + h], s_r[(6 * q + 2 * u + 1) * SHV + h]};
-      rv[pe] = pack_unit(r2);
-      rv[po] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k = 0; k < 12; ++k) f[k] += 0.5f * a[k];
+          }
+        } else {                              // minimal-residual step with p = A_ee r^ - D_eo t_o = a / 2
+          float pr = 0.f, pi = 0.f, pp = 0.f;
+          if (!p) {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+              a[k] = 0.5f * a[k];
+              pr += a[k].re * f[k].re + a[k].im * f[k].im;
+              pi += a[k].re * f[k].im - a[k].im * f[k].re;
+              pp += a[k].re * a[k].re + a[k].im * a[k].im;
+            }
+          }
+          // sum over the even sites: their warps only (one warp holds both parities when SHV = 16)
+          if (SHV < 32 || !p) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+              pr += __shfl_xor_sync(0xffffffffu, pr, o);
+              pi += __shfl_xor_sync(0xffffffffu, pi, o);
+              pp += __shfl_xor_sync(0xffffffffu, pp, o);
+            }
+            if constexpr (NW > 1) {
+              if ((t & 31) == 0) { s_red[0][t >> 5] = pr; s_red[1][t >> 5] = pi; s_red[2][t >> 5] = pp; }
+              bar_wait(2, SHV);
+              pr = 0.f; pi = 0.f; pp = 0.f;
+#pragma unroll
+              for (int j = 0; j < NW; ++j) { pr += s_red[0][j]; pi += s_red[1][j]; pp += s_red[2][j]; }
+            }
+          }
+          if (!p) {
+            cplx<float> al = {0.f, 0.f};
+            if (pp > 0.f) al = {pr / pp, pi / pp};
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+              cplx<float> x[2];
+              unpack_unit(sb.xb[k * NS + t], x);
+              cmac(x[0], al, f[2 * k]);
+              cmac(x[1], al, f[2 * k + 1]);
+              sb.xb[k * NS + t] = pack_unit(x);
+            }
+#pragma unroll
+            for (int k = 0; k < 12; ++k) cmsub(f[k], al, a[k]);
+          }
+        }
+        if (!p) {
+          if (s + 1 == last) {                // the new residual on the even sites; x_e goes on
+            if (rdst0) store_site<float, 12>(rdst0 + fo, V, i, f);
+            sb.get(sb.xb, NS, t, f);
+          }
+          sb.put(sb.vec, SHV, h, f);
+        }
+      }
+      __syncthreads();
     }
+    // f = x_e, x_o; the new residual vanishes on the odd sites
+    if (rdst0 && p) {
+#pragma unroll
+      for (int k = 0; k < 12; ++k) a[k] = {0.f, 0.f};
+      store_site<float, 12>(rdst0 + fo, V, i, a);
+    }
+    if (dout0) store_site<float, 12>(dout0 + fo, V, i, f);
     if (!first) {
-      float4 a = xv[pe], c = xv[po];
-      xe.x += a.x; xe.y += a.y; xe.z += a.z; xe.w += a.w;
-      xo.x += c.x; xo.y += c.y; xo.z += c.z; xo.w += c.w;
+      load_site_rw<float, 12>(xi0 + fo, V, i, a);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) f[k] += a[k];
     }
-    xv[pe] = xe;
-    xv[po] = xo;
+    store_site<float, 12>(xi0 + fo, V, i, f);
+    __syncthreads();             // the next right-hand side writes half, vec and xb
   }
-  __syncthreads();   // shared buffers are reused by the next right-hand side
+  if constexpr (Cfg::TM) {
+    if (t < 32)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tm), "r"((uint32_t)Cfg::TCOLS)
+                   : "memory");
   }
+}
+
+// Right-hand sides per CTA of a batch.  A CTA that takes several stages the block once for all of them,
+// but too few CTAs leave SMs idle: the number of waves times the work of a CTA is made smallest (staging
+// costs about 0.1 of a block solve).  20 fields at 24x16^3 (192 blocks of a colour, 304 CTAs resident):
+// 3.41 ms; one CTA for all fields of a block 6.86 ms with the kernel this one replaced.
+inline int sap_rhs_per_cta(int nblocks, int nrhs, int slots) {
+  int best = nrhs;
+  double best_t = 1e300;
+  for (int g = 1; g <= nrhs; ++g) {
+    const int rpc = (nrhs + g - 1) / g;
+    const long long ctas = (long long)nblocks * ((nrhs + rpc - 1) / rpc);
+    const double t = (double)((ctas + slots - 1) / slots) * (rpc + 0.1);
+    if (t < best_t * 0.999) { best_t = t; best = rpc; }
+  }
+  return best;
 }
 
 template <int SHV>
 bool launch_sap_staged(dw_ctx* c, int colour, const float* rsrc, float* rdst, const float* dprev, float* dout,
                        float* xi, int first, int nmr, cudaStream_t st, int nrhs = 1) {
-  constexpr size_t smem = (36 * 2 * SHV + 3 * 12 * SHV) * sizeof(cplx<float>);
+  constexpr size_t smem = SapCfg<SHV>::bytes;
   static int state = 0;   // 0 unknown, 1 ok, -1 unavailable
   if (state == 0) {
     cudaError_t e = cudaFuncSetAttribute(sap_staged_kernel<SHV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -490,11 +759,14 @@ bool launch_sap_staged(dw_ctx* c, int colour, const float* rsrc, float* rdst, co
   }
   if (state < 0) return false;
   const int* list = c->d_colour_list + (colour ? c->ncolour[0] : 0);
-  sap_staged_kernel<SHV><<<c->ncolour[colour], 2 * SHV, smem, st>>>(c->g, (const float*)c->links[DW_F32],
-                                                                   (const float*)c->clov[DW_F32],
-                                                                   (const float*)c->clovinv[DW_F32], list, rsrc,
-                                                                   rdst, dprev, dout, xi, first, nmr, nrhs,
-                                                                   (size_t)c->V * 24); dw_note_launch();
+  const int slots = c->sms * (256 / SHV);                                // resident CTAs (launch bounds)
+  const int rpc = sap_rhs_per_cta(c->ncolour[colour], nrhs, slots);
+  const dim3 grid((unsigned)c->ncolour[colour], (unsigned)((nrhs + rpc - 1) / rpc));
+  sap_staged_kernel<SHV><<<grid, 2 * SHV, smem, st>>>(c->g, (const float*)c->links[DW_F32],
+                                                      (const float*)c->clov[DW_F32],
+                                                      (const float*)c->clovinv[DW_F32], list, rsrc,
+                                                      rdst, dprev, dout, xi, first, nmr, nrhs, rpc,
+                                                      (size_t)c->V * 24); dw_note_launch();
   return true;
 }
 

@@ -349,6 +349,7 @@ extern "C" int dw_create(const dw_params* p, const double* links_host, dw_ctx** 
   dw_ctx* c = new dw_ctx();
   c->p = *p;
   c->device = dev;
+  cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
   {
     uint64_t h = 1469598103934665603ull;       // FNV-1a over the bytes of the canonical links
     const unsigned char* b = reinterpret_cast<const unsigned char*>(links_host);
