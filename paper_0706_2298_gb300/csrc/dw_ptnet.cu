@@ -20,7 +20,11 @@
 
 namespace {
 
-constexpr int PT_THREADS = 128;
+// Every kernel works on tiles of PT_S consecutive sites of one field, a lane per site (V is a multiple of 256:
+// Schwarz blocks have at least 16 sites and there are at least 16 of them); the tiles of all fields of a
+// batch form one grid.
+constexpr int PT_S = 32;
+constexpr int PT_THREADS = 256;
 
 // transport of one channel field along PTNet direction d (0 = none) to site s/i; out[4][3]
 DW_D void pt_transport(const Geom& g, const float* __restrict__ links, const float* __restrict__ f,
@@ -51,129 +55,286 @@ DW_D void pt_transport(const Geom& g, const float* __restrict__ links, const flo
   }
 }
 
-// one layer (ADJ = false) or its adjoint (ADJ = true); thread = (site, output channel)
-template <int CIN, int COUT, bool ADJ>
-__global__ void __launch_bounds__(PT_THREADS) ptnet_layer_kernel(Geom g, const float* __restrict__ links,
-                                                                 const float2* __restrict__ W,
-                                                                 const float* __restrict__ in,
-                                                                 float* __restrict__ out) {
-  constexpr int NI = ADJ ? COUT : CIN;      // channels read
-  constexpr int NO = ADJ ? CIN : COUT;      // channels written
-  constexpr int SPB = PT_THREADS / NO;      // sites per block
-  __shared__ float2 sW[4 * NO][4 * NI];
-  const int t = threadIdx.x;
-  const int co = t % NO, sl = t / NO;
-  const long long i = (long long)blockIdx.x * SPB + sl;
-  const bool valid = sl < SPB && i < g.V;
-  const size_t fs = (size_t)g.V * 24;
-  SiteRef s = decode(g, valid ? i : 0);
-  cplx<float> acc[4][3];
-#pragma unroll
-  for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-    for (int a = 0; a < 3; ++a) acc[sp][a] = {0.f, 0.f};
-  for (int d = 0; d < 9; ++d) {
-    __syncthreads();
-    const float2* Wd = W + (size_t)d * (4 * COUT) * (4 * CIN);
-    for (int e = t; e < 16 * NO * NI; e += PT_THREADS) {
-      const int r = e / (4 * NI), c = e % (4 * NI);
-      // forward: sW = W_d [4 COUT][4 CIN]; adjoint: sW = W_d^+ [4 CIN][4 COUT]
-      float2 w = ADJ ? Wd[(size_t)c * (4 * CIN) + r] : Wd[(size_t)r * (4 * CIN) + c];
-      sW[r][c] = ADJ ? make_float2(w.x, -w.y) : w;
-    }
-    __syncthreads();
-    if (!valid) continue;
-    // adjoint transport: T_{+mu}^+ has the form of T_{-mu} and vice versa
-    const int dt = (ADJ && d > 0) ? (((d - 1) ^ 1) + 1) : d;
-    for (int ci = 0; ci < NI; ++ci) {
-      cplx<float> th[4][3];
-      pt_transport(g, links, in + (size_t)ci * fs, s, i, dt, th);
-#pragma unroll
-      for (int so = 0; so < 4; ++so) {
-#pragma unroll
-        for (int si = 0; si < 4; ++si) {
-          const float2 w = sW[4 * co + so][4 * ci + si];
-          const cplx<float> wc = {w.x, w.y};
-#pragma unroll
-          for (int a = 0; a < 3; ++a) acc[so][a] += wc * th[si][a];
-        }
-      }
-    }
+// direction of the adjoint transport: T_{+mu}^+ has the form of T_{-mu} and vice versa
+DW_D int pt_reverse(int d) { return d > 0 ? ((d - 1) ^ 1) + 1 : 0; }
+
+struct PtTile {
+  size_t field;      // field of the batch
+  long long i;       // this lane's site
+  SiteRef s;
+  DW_D PtTile(const Geom& g, long long tile) {
+    const long long per = g.V / PT_S;
+    field = (size_t)(tile / per);
+    i = (tile % per) * PT_S + (threadIdx.x & 31);
+    s = decode(g, i);
   }
-  if (!valid) return;
-  cplx<float> o[12];
+};
+
+// NI -> 16 channels: out = sum_d W_d T_d in, or for ADJ the adjoint sum_d W_d^+ T_d^+ in of a layer with NI
+// output channels.  A complex matrix product per site and colour: 64 rows (channel, spin) written, 4 NI rows
+// read per direction.  Per stage (a direction; all nine for NI = 1) the transported input of the tile's 32
+// sites and the weights go to shared memory once, and a thread accumulates 8 rows x 3 colours of its site:
+// 96 FMAs per 4 uniform 16-byte and 3 8-byte shared-memory reads.  The sums of a direction are kept apart
+// and then added, which keeps the chains of FP32 roundings short.
+// Bound: FP32 FMA issue (885 kflop per site for NI = 16).
+template <int NI>
+struct PtLayer {
+  static constexpr int DPS = NI == 1 ? 9 : 1, NST = 9 / DPS, K = DPS * 4 * NI;
+  static constexpr int WS = 66;                              // row stride of the staged weights (bank spread)
+  static constexpr size_t bytes = (size_t)K * (WS + 3 * PT_S) * sizeof(float2);
+};
+template <int NI, bool ADJ>
+__global__ void __launch_bounds__(PT_THREADS, 2) ptnet_layer_kernel(Geom g, const float* __restrict__ links,
+                                                                    const float2* __restrict__ W,
+                                                                    const float* __restrict__ in,
+                                                                    float* __restrict__ out) {
+  using C = PtLayer<NI>;
+  extern __shared__ __align__(16) unsigned char pt_smem[];
+  float2* sW = reinterpret_cast<float2*>(pt_smem);           // [K][WS]
+  cplx<float>* sB = reinterpret_cast<cplx<float>*>(sW + C::K * C::WS);     // [K][3][PT_S]
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const PtTile tl(g, blockIdx.x);
+  const size_t fs = (size_t)g.V * 24;
+  const float* fin = in + tl.field * NI * fs;
+  cplx<float> acc[8][3];
 #pragma unroll
-  for (int sp = 0; sp < 4; ++sp)
+  for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int a = 0; a < 3; ++a) o[3 * sp + a] = acc[sp][a];
-  store_site<float, 12>(out + (size_t)co * fs, g.V, i, o);
+    for (int a = 0; a < 3; ++a) acc[r][a] = {0.f, 0.f};
+  for (int st = 0; st < C::NST; ++st) {
+    __syncthreads();
+    // weights as [k][row]: forward W_d [64][4 NI], adjoint W_d^+ of W_d [4 NI][64]
+    for (int e = t; e < C::K * 64; e += PT_THREADS) {
+      int k, r;
+      float2 w;
+      if (ADJ) {
+        k = e >> 6; r = e & 63;
+        w = W[(size_t)st * C::K * 64 + e];
+        w.y = -w.y;
+      } else {
+        const int d = e / (256 * NI), q = e % (256 * NI);      // within the stage
+        r = q / (4 * NI); k = d * 4 * NI + q % (4 * NI);
+        w = W[(size_t)st * C::K * 64 + e];
+      }
+      sW[k * C::WS + r] = w;
+    }
+    for (int it = warp; it < C::DPS * NI; it += PT_THREADS / 32) {
+      const int d = NI == 1 ? it : st, c = NI == 1 ? 0 : it;
+      cplx<float> th[4][3];
+      pt_transport(g, links, fin + (size_t)c * fs, tl.s, tl.i, ADJ ? pt_reverse(d) : d, th);
+#pragma unroll
+      for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) sB[((4 * it + sp) * 3 + a) * PT_S + lane] = th[sp][a];
+    }
+    __syncthreads();
+    cplx<float> part[8][3];
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) part[r][a] = {0.f, 0.f};
+#pragma unroll 2
+    for (int k = 0; k < C::K; ++k) {
+      cplx<float> w[8], b[3];
+      const float4* wp = reinterpret_cast<const float4*>(sW + k * C::WS + 8 * warp);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) unpack_unit(wp[q], w + 2 * q);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) b[a] = sB[(k * 3 + a) * PT_S + lane];
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) cmac(part[r][a], w[r], b[a]);
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) acc[r][a] += part[r][a];
+  }
+  // rows 8 warp .. are the two channels 2 warp, 2 warp + 1
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    store_site<float, 12>(out + (tl.field * 16 + 2 * warp + q) * fs, g.V, tl.i, &acc[4 * q][0]);
 }
 
-// partial weight gradients: CTA (chunk, d) sums g'(x) (T_d h)(x)^+ over its sites
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(256) ptnet_dw_kernel(Geom g, const float* __restrict__ links,
-                                                       const float* __restrict__ gout,
-                                                       const float* __restrict__ h, float2* partial,
-                                                       long long chunk) {
-  constexpr int S = 8;                         // sites per tile
-  constexpr int E = 16 * COUT * CIN;           // entries of W_d
-  constexpr int EPT = (E + 255) / 256;         // entries per thread
-  __shared__ cplx<float> sg[S][4 * COUT][3];
-  __shared__ cplx<float> sx[S][4 * CIN][3];
-  const int d = blockIdx.y;
-  const long long i0 = (long long)blockIdx.x * chunk, i1 = min(i0 + chunk, (long long)g.V);
+// 16 -> 1 channel layer, first half: the weights act on (channel, spin) and the transports on (site,
+// colour), so the channels are contracted before the transport: z_d = W_d h, nine fields, each
+// transported once, instead of 16 x 9 transports per site.  Rows (d, spin): 36, a warp takes two
+// directions; cols and staging as above.
+constexpr int PT_ZW = 5;                                     // warps of the contraction
+constexpr size_t PT_Z_BYTES = (size_t)64 * (40 + 3 * PT_S) * sizeof(float2);
+__global__ void __launch_bounds__(32 * PT_ZW) ptnet_contract_kernel(Geom g, const float2* __restrict__ W,
+                                                                    const float* __restrict__ in,
+                                                                    float* __restrict__ z) {
+  extern __shared__ __align__(16) unsigned char pt_smem[];
+  float2* sW = reinterpret_cast<float2*>(pt_smem);           // [64][40]
+  cplx<float>* sB = reinterpret_cast<cplx<float>*>(sW + 64 * 40);          // [64][3][PT_S]
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const PtTile tl(g, blockIdx.x);
   const size_t fs = (size_t)g.V * 24;
-  // per entry: the sum of a tile (S sites x 3 colours, 24 products) is formed in FP32 and
-  // folded into a compensated (Kahan) FP32 accumulator, so that the error of a chunk's sum does
-  // not grow with the number of sites it covers
-  cplx<float> acc[EPT], cmp[EPT];
+  for (int e = t; e < 64 * 40; e += 32 * PT_ZW) {
+    const int r = e >> 6, k = e & 63;                        // row (d, spin) of W [9][4][64]
+    sW[k * 40 + r] = r < 36 ? W[r * 64 + k] : make_float2(0.f, 0.f);
+  }
+  for (int c = warp; c < 16; c += PT_ZW) {
+    cplx<float> p[12];
+    load_site<float, 12>(in + (tl.field * 16 + c) * fs, g.V, tl.i, p);
 #pragma unroll
-  for (int k = 0; k < EPT; ++k) { acc[k] = {0.f, 0.f}; cmp[k] = {0.f, 0.f}; }
-  for (long long b0 = i0; b0 < i1; b0 += S) {
+    for (int k = 0; k < 12; ++k) sB[((4 * c + k / 3) * 3 + k % 3) * PT_S + lane] = p[k];
+  }
+  __syncthreads();
+  cplx<float> acc[8][3];
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) acc[r][a] = {0.f, 0.f};
+#pragma unroll 2
+  for (int k = 0; k < 64; ++k) {
+    cplx<float> w[8], b[3];
+    const float4* wp = reinterpret_cast<const float4*>(sW + k * 40 + 8 * warp);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) unpack_unit(wp[q], w + 2 * q);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) b[a] = sB[(k * 3 + a) * PT_S + lane];
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) cmac(acc[r][a], w[r], b[a]);
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    if (2 * warp + q < 9)
+      store_site<float, 12>(z + (tl.field * 9 + 2 * warp + q) * fs, g.V, tl.i, &acc[4 * q][0]);
+}
+// second half: out = sum_d T_d z_d; a thread per site
+__global__ void __launch_bounds__(128) ptnet_collect_kernel(Geom g, const float* __restrict__ links,
+                                                            const float* __restrict__ z, float* __restrict__ out) {
+  const long long t = blockIdx.x * 128LL + threadIdx.x;
+  const size_t f = (size_t)(t / g.V), fs = (size_t)g.V * 24;   // V is a multiple of 128
+  const long long i = t % g.V;
+  const SiteRef s = decode(g, i);
+  cplx<float> acc[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = {0.f, 0.f};
+#pragma unroll
+  for (int d = 0; d < 9; ++d) {
+    cplx<float> th[4][3];
+    pt_transport(g, links, z + (f * 9 + d) * fs, s, i, d, th);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] += th[k / 3][k % 3];
+  }
+  store_site<float, 12>(out + f * fs, g.V, i, acc);
+}
+
+// Partial weight gradients dW_d = sum_{x, colour} g(x) (T_d h)(x)^+ over a chunk of tiles.  A CTA forms
+// A B^+ with A: 64 rows (16 channels x spin) of a field taken where it stands, B: transported rows.
+//   MODE 0 (16 -> 16): A = g, B = T_d h of direction d = blockIdx.y (64 rows)
+//   MODE 1 (1 -> 16):  A = g, B = (T_0 h .. T_8 h) of the single input channel (36 rows)
+//   MODE 2 (16 -> 1):  A = h, B = (T_0^+ g .. T_8^+ g) of the single output channel (36 rows); the sum over
+//                      sites moved by the transport, g (T_d h)^+ = (T_d^+ g) h^+, so that one field is
+//                      transported instead of 16; the entries are conjugated and transposed
+// A thread owns 4 x 4 entries.  Per entry the sum of 8 sites (24 products) is formed in FP32 and folded into
+// a compensated (Kahan) FP32 accumulator, so that the error of a chunk's sum does not grow with the number
+// of sites it covers.
+constexpr int PT_K = 3 * PT_S;                               // (site, colour) per tile
+constexpr int PT_AS = 66;
+template <int MODE>
+struct PtDw {
+  static constexpr int N = MODE == 0 ? 64 : 36, BS = N + 2;
+  static constexpr size_t bytes = (size_t)PT_K * (PT_AS + BS) * sizeof(float2);
+};
+template <int MODE>
+__global__ void __launch_bounds__(PT_THREADS, 2) ptnet_dw_kernel(Geom g, const float* __restrict__ links,
+                                                                 const float* __restrict__ local,
+                                                                 const float* __restrict__ moved, float2* partial,
+                                                                 long long ntiles) {
+  using C = PtDw<MODE>;
+  constexpr int NC = C::N / 4;                               // column groups
+  extern __shared__ __align__(16) unsigned char pt_smem[];
+  cplx<float>* sA = reinterpret_cast<cplx<float>*>(pt_smem); // [PT_K][PT_AS]
+  cplx<float>* sB = sA + PT_K * PT_AS;                       // [PT_K][BS]
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int tr = t / NC, tc = t - tr * NC;
+  const bool active = tr < 16;
+  const size_t fs = (size_t)g.V * 24;
+  cplx<float> acc[4][4], cmp[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) { acc[r][c] = {0.f, 0.f}; cmp[r][c] = {0.f, 0.f}; }
+  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const PtTile tl(g, tile);
     __syncthreads();
-    for (int w = threadIdx.x; w < S * (COUT + CIN); w += 256) {
-      const int sl = w % S, job = w / S;
-      const long long i = b0 + sl;
-      if (i >= i1) {
-        if (job < COUT) { for (int r = 0; r < 4; ++r) for (int a = 0; a < 3; ++a) sg[sl][4 * job + r][a] = {0.f, 0.f}; }
-        else { const int c = job - COUT; for (int r = 0; r < 4; ++r) for (int a = 0; a < 3; ++a) sx[sl][4 * c + r][a] = {0.f, 0.f}; }
-        continue;
-      }
-      if (job < COUT) {
-        cplx<float> p[12];
-        load_site<float, 12>(gout + (size_t)job * fs, g.V, i, p);
-        for (int r = 0; r < 4; ++r) for (int a = 0; a < 3; ++a) sg[sl][4 * job + r][a] = p[3 * r + a];
-      } else {
-        const int c = job - COUT;
-        cplx<float> th[4][3];
-        SiteRef s = decode(g, i);
-        pt_transport(g, links, h + (size_t)c * fs, s, i, d, th);
-        for (int r = 0; r < 4; ++r) for (int a = 0; a < 3; ++a) sx[sl][4 * c + r][a] = th[r][a];
-      }
+    for (int c = warp; c < 16; c += PT_THREADS / 32) {
+      cplx<float> p[12];
+      load_site<float, 12>(local + (tl.field * 16 + c) * fs, g.V, tl.i, p);
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int sp = 0; sp < 4; sp += 2) {
+          const cplx<float> v[2] = {p[3 * sp + a], p[3 * (sp + 1) + a]};
+          *reinterpret_cast<float4*>(sA + (3 * lane + a) * PT_AS + 4 * c + sp) = pack_unit(v);
+        }
+    }
+    for (int it = warp; it < NC; it += PT_THREADS / 32) {    // it: channel (MODE 0) or direction
+      const int d = MODE == 0 ? (int)blockIdx.y : MODE == 1 ? it : pt_reverse(it);
+      const float* f = moved + (MODE == 0 ? tl.field * 16 + it : tl.field) * fs;
+      cplx<float> th[4][3];
+      pt_transport(g, links, f, tl.s, tl.i, d, th);
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int sp = 0; sp < 4; sp += 2) {
+          const cplx<float> v[2] = {th[sp][a], th[sp + 1][a]};
+          *reinterpret_cast<float4*>(sB + (3 * lane + a) * C::BS + 4 * it + sp) = pack_unit(v);
+        }
     }
     __syncthreads();
+    if (active) {
+      for (int k0 = 0; k0 < PT_K; k0 += 24) {
+        cplx<float> part[4][4];
 #pragma unroll
-    for (int k = 0; k < EPT; ++k) {
-      const int e = threadIdx.x + 256 * k;
-      if (e < E) {
-        const int r = e / (4 * CIN), c = e % (4 * CIN);
-        cplx<float> tile = {0.f, 0.f};
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int sl = 0; sl < S; ++sl)
+          for (int c = 0; c < 4; ++c) part[r][c] = {0.f, 0.f};
+#pragma unroll 4
+        for (int k = k0; k < k0 + 24; ++k) {
+          cplx<float> av[4], bv[4];
+          const float4* ap = reinterpret_cast<const float4*>(sA + k * PT_AS + 4 * tr);
+          const float4* bp = reinterpret_cast<const float4*>(sB + k * C::BS + 4 * tc);
+          unpack_unit(ap[0], av);
+          unpack_unit(ap[1], av + 2);
+          unpack_unit(bp[0], bv);
+          unpack_unit(bp[1], bv + 2);
 #pragma unroll
-          for (int a = 0; a < 3; ++a) tile += cmulc(sx[sl][c][a], sg[sl][r][a]);
-        const float yr = tile.re - cmp[k].re, yi = tile.im - cmp[k].im;
-        const float tr = acc[k].re + yr, tq = acc[k].im + yi;
-        cmp[k] = {(tr - acc[k].re) - yr, (tq - acc[k].im) - yi};
-        acc[k] = {tr, tq};
+          for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) cmacc(part[r][c], bv[c], av[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const float yr = part[r][c].re - cmp[r][c].re, yi = part[r][c].im - cmp[r][c].im;
+            const float sr = acc[r][c].re + yr, si = acc[r][c].im + yi;
+            cmp[r][c] = {(sr - acc[r][c].re) - yr, (si - acc[r][c].im) - yi};
+            acc[r][c] = {sr, si};
+          }
       }
     }
   }
+  if (!active) return;
+  // [chunk][d][entry], entries as in the weights
 #pragma unroll
-  for (int k = 0; k < EPT; ++k) {
-    const int e = threadIdx.x + 256 * k;
-    if (e < E) partial[((size_t)blockIdx.x * 9 + d) * E + e] = make_float2(acc[k].re, acc[k].im);
-  }
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int row = 4 * tr + r;
+      const float2 v = make_float2(acc[r][c].re, MODE == 2 ? -acc[r][c].im : acc[r][c].im);
+      if (MODE == 0) partial[((size_t)blockIdx.x * 9 + blockIdx.y) * 4096 + row * 64 + 4 * tc + c] = v;
+      else if (MODE == 1) partial[((size_t)blockIdx.x * 9 + tc) * 256 + row * 4 + c] = v;
+      else partial[((size_t)blockIdx.x * 9 + tc) * 256 + c * 64 + row] = v;
+    }
 }
 
 // grad[d][e] = scale * sum over chunks (fixed order)
@@ -203,13 +364,55 @@ __global__ void ptnet_adam_kernel(size_t n, float* w, const float* gr, float* m,
   w[t] -= lr * (mt / c1) / (sqrtf(vt / c2) + eps);
 }
 
-template <int CIN, int COUT, bool ADJ>
-void launch_layer(dw_ctx* c, const float2* W, const float* in, float* out, cudaStream_t st) {
-  constexpr int NO = ADJ ? CIN : COUT;
-  constexpr int SPB = PT_THREADS / NO;
-  const unsigned blocks = (unsigned)((c->V + SPB - 1) / SPB);
-  ptnet_layer_kernel<CIN, COUT, ADJ><<<blocks, PT_THREADS, 0, st>>>(c->g, (const float*)c->links[DW_F32], W, in,
-                                                                    out); dw_note_launch();
+// dynamic shared memory of a kernel above the 48 KB default, once per kernel
+template <typename F>
+cudaError_t pt_attr(F* f, size_t bytes) {
+  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+// nf fields: NI channels each in, 16 out (ADJ: the adjoint of a 16 -> NI layer)
+template <int NI, bool ADJ>
+cudaError_t launch_layer(dw_ctx* c, const float2* W, const float* in, float* out, int nf, cudaStream_t st) {
+  static const cudaError_t attr = pt_attr(ptnet_layer_kernel<NI, ADJ>, PtLayer<NI>::bytes);
+  if (attr != cudaSuccess) return attr;
+  const unsigned tiles = (unsigned)(c->V / PT_S * nf);
+  ptnet_layer_kernel<NI, ADJ><<<tiles, PT_THREADS, PtLayer<NI>::bytes, st>>>(c->g, (const float*)c->links[DW_F32], W,
+                                                                             in, out);
+  dw_note_launch();
+  return cudaGetLastError();
+}
+// 16 channels in, 1 out; z: 9 scratch fields per field
+cudaError_t launch_layer_last(dw_ctx* c, const float2* W, const float* in, float* z, float* out, int nf,
+                              cudaStream_t st) {
+  static const cudaError_t attr = pt_attr(ptnet_contract_kernel, PT_Z_BYTES);
+  if (attr != cudaSuccess) return attr;
+  ptnet_contract_kernel<<<(unsigned)(c->V / PT_S * nf), 32 * PT_ZW, PT_Z_BYTES, st>>>(c->g, W, in, z);
+  dw_note_launch();
+  ptnet_collect_kernel<<<(unsigned)(c->V / 128 * nf), 128, 0, st>>>(c->g, (const float*)c->links[DW_F32], z, out);
+  dw_note_launch();
+  return cudaGetLastError();
+}
+// CTAs over the tiles of a weight gradient: two waves of the resident CTAs (two per SM) in all directions
+int pt_chunks(const dw_ctx* c, long long tiles, int ndir) {
+  return (int)std::min<long long>(tiles, std::max(1, 4 * c->sms / ndir));
+}
+template <int MODE>
+cudaError_t launch_dw(dw_ctx* c, const float* local, const float* moved, float2* partial, float2* grad, int nf,
+                      cudaStream_t st) {
+  static const cudaError_t attr = pt_attr(ptnet_dw_kernel<MODE>, PtDw<MODE>::bytes);
+  if (attr != cudaSuccess) return attr;
+  constexpr int E = MODE == 0 ? 4096 : 256, ND = MODE == 0 ? 9 : 1;
+  const long long tiles = c->V / PT_S * nf;
+  const int nc = pt_chunks(c, tiles, ND);
+  ptnet_dw_kernel<MODE><<<dim3(nc, ND), PT_THREADS, PtDw<MODE>::bytes, st>>>(c->g, (const float*)c->links[DW_F32],
+                                                                             local, moved, partial, tiles);
+  dw_note_launch();
+  ptnet_dw_reduce_kernel<<<(unsigned)((9 * E + 255) / 256), 256, 0, st>>>(partial, nc, E, 2.f, grad);
+  dw_note_launch();
+  return cudaGetLastError();
+}
+// fields worked on together: enough for a full GPU, at most 2^19 sites (about 3.7 GB of training workspace)
+int pt_group(const dw_ctx* c, int nf) {
+  return (int)std::min<long long>(nf, std::max<long long>(1, (1LL << 19) / c->V));
 }
 
 // ------------------------------------------------------------------ tensor-core 16 -> 16 layer
@@ -489,28 +692,14 @@ extern "C" size_t ptnet_weight_count(int C) {
 
 static bool ptnet_ok(int C) { return C == 16; }
 
-// acts: 2 * C fields (the two hidden layers), may be null for inference
-static int ptnet_forward_impl(dw_ctx* c, int C, const float2* W, const float* x, float* y, float* acts,
-                              cudaStream_t st) {
-  const size_t fs = (size_t)c->V * 24;
-  float* h1 = acts;
-  float* own = nullptr;
-  if (!h1) {
-    DW_CUDA(cudaMalloc(&own, 2 * C * fs * sizeof(float)));
-    h1 = own;
-  }
-  float* h2 = h1 + (size_t)C * fs;
-  const size_t w1 = 9 * 16 * C, w2 = 9 * 16 * C * C;
-  launch_layer<1, 16, false>(c, W, x, h1, st);
-  launch_layer<16, 16, false>(c, W + w1, h1, h2, st);
-  launch_layer<16, 1, false>(c, W + w1 + w2, h2, y, st);
-  cudaError_t e = cudaGetLastError();
-  if (own) {
-    cudaStreamSynchronize(st);
-    cudaFree(own);
-  }
-  if (e != cudaSuccess) return dw_cuda_fail(e, "ptnet_forward");
-  return DW_OK;
+// y = N(x) for nf fields (one batch); h1, h2: 16 fields per field, z: 9 per field (h1 where it is not needed later)
+static cudaError_t ptnet_forward_impl(dw_ctx* c, const float2* W, const float* x, float* y, float* h1, float* h2,
+                                      float* z, int nf, cudaStream_t st) {
+  const size_t w1 = 9 * 16 * 16, w2 = w1 * 16;
+  cudaError_t e = launch_layer<1, false>(c, W, x, h1, nf, st);
+  if (e == cudaSuccess) e = launch_layer<16, false>(c, W + w1, h1, h2, nf, st);
+  if (e == cudaSuccess) e = launch_layer_last(c, W + w1 + w2, h2, z, y, nf, st);
+  return e;
 }
 
 extern "C" int ptnet_forward(dw_ctx* c, int C, const void* W, int nf, const void* x, void* y, void* stream) {
@@ -519,15 +708,19 @@ extern "C" int ptnet_forward(dw_ctx* c, int C, const void* W, int nf, const void
     return DW_EINVAL;
   }
   const size_t fs = (size_t)c->V * 24;
+  const int ng = pt_group(c, nf);
   float* acts = nullptr;
-  DW_CUDA(cudaMalloc(&acts, 2 * C * fs * sizeof(float)));
-  int rc = DW_OK;
-  for (int f = 0; f < nf && rc == DW_OK; ++f)
-    rc = ptnet_forward_impl(c, C, (const float2*)W, (const float*)x + f * fs, (float*)y + f * fs, acts,
-                            (cudaStream_t)stream);
-  cudaStreamSynchronize((cudaStream_t)stream);
+  DW_CUDA(cudaMalloc(&acts, 2 * C * fs * ng * sizeof(float)));
+  cudaError_t e = cudaSuccess;
+  for (int f = 0; f < nf && e == cudaSuccess; f += ng) {
+    const int n = std::min(ng, nf - f);
+    e = ptnet_forward_impl(c, (const float2*)W, (const float*)x + f * fs, (float*)y + f * fs, acts,
+                           acts + (size_t)C * fs * ng, acts, n, (cudaStream_t)stream);
+  }
+  const cudaError_t es = cudaStreamSynchronize((cudaStream_t)stream);
   cudaFree(acts);
-  return rc;
+  if (e == cudaSuccess) e = es;
+  return e == cudaSuccess ? DW_OK : dw_cuda_fail(e, "ptnet_forward");
 }
 
 // One 16 -> 16 layer on a set of 16 channel fields: out = sum_d W_d T_d in (adjoint:
@@ -538,9 +731,8 @@ extern "C" int ptnet_layer16(dw_ctx* c, const void* W, int adjoint, int tensor_c
   if (int rc = dw_check_device(c, "ptnet_layer16")) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   if (tensor_cores) return tc_layer16(c, (const float2*)W, adjoint, (const float*)in, (float*)out, st);
-  if (adjoint) launch_layer<16, 16, true>(c, (const float2*)W, (const float*)in, (float*)out, st);
-  else launch_layer<16, 16, false>(c, (const float2*)W, (const float*)in, (float*)out, st);
-  DW_CUDA(cudaGetLastError());
+  DW_CUDA(adjoint ? (launch_layer<16, true>(c, (const float2*)W, (const float*)in, (float*)out, 1, st))
+                  : (launch_layer<16, false>(c, (const float2*)W, (const float*)in, (float*)out, 1, st)));
   DW_CUDA(cudaStreamSynchronize(st));
   return DW_OK;
 }
@@ -562,9 +754,12 @@ extern "C" int ptnet_forward_tc(dw_ctx* c, int C, const void* Wv, int nf, const 
   float* h2 = acts + (size_t)C * fs;
   int rc = DW_OK;
   for (int f = 0; f < nf && rc == DW_OK; ++f) {
-    launch_layer<1, 16, false>(c, W, (const float*)x + f * fs, h1, st);
-    rc = tc_layer16(c, W + w1, 0, h1, h2, st);
-    if (rc == DW_OK) launch_layer<16, 1, false>(c, W + w1 + w2, h2, (float*)y + f * fs, st);
+    cudaError_t e = launch_layer<1, false>(c, W, (const float*)x + f * fs, h1, 1, st);
+    if (e == cudaSuccess) {
+      rc = tc_layer16(c, W + w1, 0, h1, h2, st);
+      if (rc == DW_OK) e = launch_layer_last(c, W + w1 + w2, h2, h1, (float*)y + f * fs, 1, st);
+    }
+    if (e != cudaSuccess) rc = dw_cuda_fail(e, "ptnet_forward_tc");
   }
   cudaStreamSynchronize(st);
   cudaFree(acts);
@@ -583,68 +778,60 @@ extern "C" int ptnet_loss_grad(dw_ctx* c, int C, const void* Wv, int nf, const v
   const float2* W = (const float2*)Wv;
   const size_t fs = (size_t)c->V * 24, n = (size_t)c->V * 12;
   const size_t w1 = 9 * 16 * C, w2 = 9 * 16 * C * C, w3 = 9 * 16 * C, nw = w1 + w2 + w3;
-  const long long chunk = 4096;
-  const int nchunk = (int)((c->V + chunk - 1) / chunk);
-  float *acts = nullptr, *out = nullptr, *g2 = nullptr, *g1 = nullptr;
-  float2 *partial = nullptr, *gacc = nullptr, *gtmp = nullptr;
-  std::vector<void*> owned;
-  auto al = [&](void** p, size_t b) -> int {
-    cudaError_t e = cudaMalloc(p, b);
-    if (e != cudaSuccess) return dw_cuda_fail(e, "cudaMalloc");
-    owned.push_back(*p);
-    return DW_OK;
-  };
-  int rc;
-  if ((rc = al((void**)&acts, 2 * C * fs * sizeof(float))) || (rc = al((void**)&out, fs * sizeof(float))) ||
-      (rc = al((void**)&g2, C * fs * sizeof(float))) || (rc = al((void**)&g1, C * fs * sizeof(float))) ||
-      (rc = al((void**)&partial, (size_t)nchunk * 9 * 16 * C * C * sizeof(float2))) ||
-      (rc = al((void**)&gacc, nw * sizeof(float2))) || (rc = al((void**)&gtmp, nw * sizeof(float2)))) {
-    for (void* p : owned) cudaFree(p);
-    return rc;
-  }
-  float* h1 = acts;
-  float* h2 = acts + (size_t)C * fs;
+  const int ng = pt_group(c, nf);
+  const size_t np = (size_t)std::max(pt_chunks(c, c->V / PT_S * ng, 9) * 9 * 4096,
+                                     pt_chunks(c, c->V / PT_S * ng, 1) * 9 * 256);
+  // the workspace stays in the context up to 8 GB: h1, h2, g2, g1 (16 fields each), the output, the gradients
+  WsArena& ar = c->ws_solve[4];
+  ar.rewind();
+  struct Keep {
+    WsArena& a;
+    bool keep;
+    ~Keep() { if (!keep) a.release(); }
+  } guard{ar, (4 * C + 1) * fs * ng * sizeof(float) <= (size_t)8 << 30};
+  float *ws = nullptr, *gw = nullptr;
+  DW_CUDA(ar.get((4 * C + 1) * fs * ng * sizeof(float), (void**)&ws));
+  DW_CUDA(ar.get((np + 2 * nw) * sizeof(float2), (void**)&gw));
+  float* h1 = ws;
+  float* h2 = h1 + (size_t)C * fs * ng;
+  float* g2 = h2 + (size_t)C * fs * ng;
+  float* g1 = g2 + (size_t)C * fs * ng;
+  float* out = g1 + (size_t)C * fs * ng;
+  float2* gacc = reinterpret_cast<float2*>(gw);
+  float2* gtmp = gacc + nw;
+  float2* partial = gtmp + nw;
   DW_CUDA(cudaMemsetAsync(gacc, 0, nw * sizeof(float2), st));
   double num = 0, den = 0;
-  std::vector<double> hh(3);
-  for (int f = 0; f < nf; ++f) {
+  double* dres = c->d_red + 65536 + 12288;
+  for (int f = 0; f < nf; f += ng) {
+    const int m = std::min(ng, nf - f);
     const float* x = (const float*)xv + f * fs;
     const float* y = (const float*)yv + f * fs;
-    if ((rc = ptnet_forward_impl(c, C, W, x, out, acts, st))) break;
-    // e = out - y ; loss numerator |e|^2, denominator |y|^2
-    blas_axpy<float>(y, out, -1.0, 0.0, n, st);
-    double* dres = c->d_red + 65536 + 12288;
-    blas_dot<float>(c, out, out, n, dres, st);
-    blas_dot<float>(c, y, y, n, dres + 3, st);
-    // back-propagation: gradient of |e|^2 wrt the output is 2 e
-    const dim3 g3(nchunk, 9);
-    ptnet_dw_kernel<16, 1><<<g3, 256, 0, st>>>(c->g, (const float*)c->links[DW_F32], out, h2, partial, chunk); dw_note_launch();
-    ptnet_dw_reduce_kernel<<<(unsigned)((9 * 16 * C + 255) / 256), 256, 0, st>>>(partial, nchunk, 16 * C, 2.f,
-                                                                               gtmp + w1 + w2); dw_note_launch();
-    launch_layer<16, 1, true>(c, W + w1 + w2, out, g2, st);
-    ptnet_dw_kernel<16, 16><<<g3, 256, 0, st>>>(c->g, (const float*)c->links[DW_F32], g2, h1, partial, chunk); dw_note_launch();
-    ptnet_dw_reduce_kernel<<<(unsigned)((9 * 16 * C * C + 255) / 256), 256, 0, st>>>(partial, nchunk, 16 * C * C,
-                                                                                   2.f, gtmp + w1); dw_note_launch();
-    launch_layer<16, 16, true>(c, W + w1, g2, g1, st);
-    ptnet_dw_kernel<1, 16><<<g3, 256, 0, st>>>(c->g, (const float*)c->links[DW_F32], g1, x, partial, chunk); dw_note_launch();
-    ptnet_dw_reduce_kernel<<<(unsigned)((9 * 16 * C + 255) / 256), 256, 0, st>>>(partial, nchunk, 16 * C, 2.f,
-                                                                               gtmp); dw_note_launch();
+    cudaError_t e = ptnet_forward_impl(c, W, x, out, h1, h2, g1, m, st);
+    if (e != cudaSuccess) return dw_cuda_fail(e, "ptnet_loss_grad");
+    // e = out - y ; loss numerator |e|^2, denominator |y|^2 (the fields of the group are contiguous)
+    blas_axpy<float>(y, out, -1.0, 0.0, n * m, st);
+    blas_dot<float>(c, out, out, n * m, dres, st);
+    blas_dot<float>(c, y, y, n * m, dres + 3, st);
+    // back-propagation: gradient of |e|^2 wrt the output is 2 e (the factor is in the reductions)
+    if ((e = launch_dw<2>(c, h2, out, partial, gtmp + w1 + w2, m, st)) != cudaSuccess ||
+        (e = launch_layer<1, true>(c, W + w1 + w2, out, g2, m, st)) != cudaSuccess ||
+        (e = launch_dw<0>(c, g2, h1, partial, gtmp + w1, m, st)) != cudaSuccess ||
+        (e = launch_layer<16, true>(c, W + w1, g2, g1, m, st)) != cudaSuccess ||
+        (e = launch_dw<1>(c, g1, x, partial, gtmp, m, st)) != cudaSuccess)
+      return dw_cuda_fail(e, "ptnet_loss_grad");
     blas_axpy<float>((const float*)gtmp, (float*)gacc, 1.0, 0.0, nw, st);
-    cudaError_t e = cudaMemcpyAsync(c->h_red, dres, 6 * sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) { rc = dw_cuda_fail(e, "ptnet_loss_grad"); break; }
+    DW_CUDA(cudaMemcpyAsync(c->h_red, dres, 6 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    DW_CUDA(cudaStreamSynchronize(st));
     num += c->h_red[2];
     den += c->h_red[5];
   }
-  if (!rc) {
-    // normalise by sum |y|^2
-    blas_scale<float>((float*)gacc, den > 0 ? 1.0 / den : 0.0, 0.0, nw, st);
-    cudaMemcpyAsync(gradv, gacc, nw * sizeof(float2), cudaMemcpyDeviceToDevice, st);
-    cudaStreamSynchronize(st);
-    if (loss) *loss = den > 0 ? num / den : 0.0;
-  }
-  for (void* p : owned) cudaFree(p);
-  return rc;
+  // normalise by sum |y|^2
+  blas_scale<float>((float*)gacc, den > 0 ? 1.0 / den : 0.0, 0.0, nw, st);
+  DW_CUDA(cudaMemcpyAsync(gradv, gacc, nw * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+  DW_CUDA(cudaStreamSynchronize(st));
+  if (loss) *loss = den > 0 ? num / den : 0.0;
+  return DW_OK;
 }
 
 extern "C" int ptnet_adam(size_t ncomplex, void* W, const void* grad, void* m, void* v, int step, double lr,
