@@ -466,16 +466,6 @@ DW_D dd split_double(double x) {
   const float lo = __uint2float_rn((unsigned)(b & 0x1FFFFFFFull)) * __uint_as_float((unsigned)(e - 948) << 23);
   return {hi, sign ? -lo : lo};
 }
-// FP32 -> FP64 by moving exponent and fraction (exact); zero and subnormal/special values aside
-DW_D double widen(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned e = (u >> 23) & 0xFFu;
-  if ((u & 0x7FFFFFFFu) == 0) return __longlong_as_double((long long)((unsigned long long)u << 32));
-  if (e == 0 || e == 255) return (double)f;
-  return __longlong_as_double((long long)(((unsigned long long)(u & 0x80000000u) << 32) |
-                                          ((unsigned long long)(e + 896) << 52) |
-                                          ((unsigned long long)(u & 0x7FFFFFu) << 29)));
-}
 
 __global__ void f64_to_dd_kernel(const double2* __restrict__ x, float4* __restrict__ y, size_t n2) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
@@ -513,11 +503,26 @@ void dd_to_f64(const dd* x, double* y, size_t n_real, int add, cudaStream_t s) {
 
 int dw_make_dd(dw_ctx* c, cudaStream_t s) {
   if (c->links_dd) return DW_OK;
-  const size_t nl = (size_t)c->V * 4 * 12, nc = (size_t)c->V * 72;   // reals (FP64 layouts)
-  DW_CUDA(cudaMalloc(&c->links_dd, nl * sizeof(dd)));
+  const size_t V = c->V, nc = V * 72;   // reals of the links (three rows) and of the clover term
+  DW_CUDA(cudaMalloc(&c->links_dd, nc * sizeof(dd)));
   DW_CUDA(cudaMalloc(&c->clov_dd, nc * sizeof(dd)));
-  f64_to_dd((const double*)c->links[DW_F64], (dd*)c->links_dd, nl, s);
+  f64_to_dd((const double*)c->links[DW_F64], (dd*)c->links_dd, nc, s);
   f64_to_dd((const double*)c->clov[DW_F64], (dd*)c->clov_dd, nc, s);
   DW_CUDA(cudaGetLastError());
   return DW_OK;
+}
+
+cudaError_t dw_pool_alloc(dw_ctx* c, size_t bytes, void** p, cudaStream_t s) {
+  if (!c->pool) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = c->device;
+    cudaError_t e = cudaMemPoolCreate(&c->pool, &props);
+    if (e != cudaSuccess) return e;
+    uint64_t keep = std::max<uint64_t>((uint64_t)4 * c->V * 24 * sizeof(double), 64u << 20);   // a pool grows by 32 MB
+    e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaMallocFromPoolAsync(p, bytes, c->pool, s);
 }

@@ -14,7 +14,7 @@
 //
 // Per-site data are stored as structure of arrays in 16-byte units:
 //   quark field : 12 complex  (k = 3*spin + colour)  -> 12*8/16 units (FP32: 6 float4, FP64: 12 double2)
-//   link        : rows 0 and 1 of U_mu(x) (6 complex), row 2 rebuilt as conj(row0 x row1)
+//   link        : FP32: rows 0 and 1 of U_mu(x) (6 complex), row 2 rebuilt as conj(row0 x row1); FP64: 9 complex
 //   clover      : per chiral 6x6 Hermitian block 18 complex slots
 //                 (slots 0..2 = real diagonal pairs, 3..17 = upper triangle row-major)
 // Unit u of site i lives at plane u: base[u * V + i], so a warp touching 32
@@ -127,6 +127,16 @@ DW_D void cmac(cplx<dd>& acc, cplx<dd> a, cplx<dd> b) { acc += a * b; }
 DW_D void cmsub(cplx<dd>& acc, cplx<dd> a, cplx<dd> b) { acc -= a * b; }
 DW_D void cmacc(cplx<dd>& acc, cplx<dd> a, cplx<dd> b) { acc += cmulc(a, b); }
 DW_D double dd_to_double(dd a) { return (double)a.hi + (double)a.lo; }
+// FP32 -> FP64 by moving exponent and fraction (exact); zero and subnormal/special values aside
+DW_D double widen(float f) {
+  const unsigned u = __float_as_uint(f);
+  const unsigned e = (u >> 23) & 0xFFu;
+  if ((u & 0x7FFFFFFFu) == 0) return __longlong_as_double((long long)((unsigned long long)u << 32));
+  if (e == 0 || e == 255) return (double)f;
+  return __longlong_as_double((long long)(((unsigned long long)(u & 0x80000000u) << 32) |
+                                          ((unsigned long long)(e + 896) << 52) |
+                                          ((unsigned long long)(u & 0x7FFFFFu) << 29)));
+}
 DW_D dd __shfl_xor_sync(unsigned mask, dd v, int lane) {
   return {__shfl_xor_sync(mask, v.hi, lane), __shfl_xor_sync(mask, v.lo, lane)};
 }
@@ -216,21 +226,29 @@ template <typename T>
 struct SU3 {
   cplx<T> m[3][3];
 };
+// FP32 links are read as two rows and the third is rebuilt; FP64 links are stored with all three: rebuilding
+// one costs 24 of the 165 FP64 instructions of a hop, the FP64 kernels run at that pipe's rate (95% of it)
+// and use a tenth of the memory bandwidth (even-odd operator at 32x16^3: 366 us with two rows).
+template <typename T> DW_HD constexpr int link_cplx() { return sizeof(T) == 8 ? 9 : 6; }
 template <typename T>
 DW_D void load_link(const T* __restrict__ links, size_t V, int mu, size_t i, SU3<T>& U) {
-  cplx<T> r[6];
-  load_site<T, 6>(links + (size_t)mu * 12 * V, V, i, r);
+  constexpr int N = link_cplx<T>();
+  cplx<T> r[N];
+  load_site<T, N>(links + (size_t)mu * 2 * N * V, V, i, r);
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     U.m[0][j] = r[j];
     U.m[1][j] = r[3 + j];
+    if constexpr (N == 9) U.m[2][j] = r[6 + j];
   }
+  if constexpr (N == 6) {
 #pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    int j1 = (j + 1) % 3, j2 = (j + 2) % 3;
-    cplx<T> r2 = U.m[0][j1] * U.m[1][j2];
-    cmsub(r2, U.m[0][j2], U.m[1][j1]);
-    U.m[2][j] = conjg(r2);
+    for (int j = 0; j < 3; ++j) {
+      int j1 = (j + 1) % 3, j2 = (j + 2) % 3;
+      cplx<T> r2 = U.m[0][j1] * U.m[1][j2];
+      cmsub(r2, U.m[0][j2], U.m[1][j1]);
+      U.m[2][j] = conjg(r2);
+    }
   }
 }
 template <typename T>
@@ -385,7 +403,7 @@ struct dw_ctx {
   void* links[2] = {nullptr, nullptr};    // [DW_F64], [DW_F32]
   void* clov[2] = {nullptr, nullptr};
   void* clovinv[2] = {nullptr, nullptr};
-  void* links_dd = nullptr;               // double-float copies (made on first use)
+  void* links_dd = nullptr;               // double-float copies (made on first use), links with three rows
   void* clov_dd = nullptr;
   void* sap_r[2] = {nullptr, nullptr};    // SAP residual workspace
   void* sap_d[2] = {nullptr, nullptr};    // SAP last-correction workspace
@@ -393,6 +411,7 @@ struct dw_ctx {
   int tune_rgroup = 0;                    // multi-RHS D variant: 0 interleaved, 1..3 per pass (autotuned)
   int tune_sap_staged = 1;                // 1: staged FP32 Schwarz kernel, 0: generic kernel (autotuned)
   void* graph_cache = nullptr;            // captured M_sap launch sequences (dw_sap.cu)
+  cudaMemPool_t pool = nullptr;           // stream-ordered scratch of calls (dw_pool_alloc)
   cudaStream_t cap_stream = nullptr;      // stream used only for graph capture
   double* d_red = nullptr;                // reduction scratch
   unsigned* d_count = nullptr;
@@ -400,6 +419,12 @@ struct dw_ctx {
   WsArena ws_solve[5];                    // solver workspaces: [0] GCR, [1] batched GCR, [2] CGNR and
                                           // BiCGstab, [3] low-mode subspace iteration, [4] network training
 };
+
+// Scratch memory of one call, stream-ordered (free it with cudaFreeAsync on the same stream).  It comes from a
+// pool of the context that keeps up to four FP64 fields (or 64 MB) between calls: with the device's default pool every
+// synchronisation returns the memory to the driver and the next call maps it again (0.5 ms).  The pool goes
+// with dw_release_workspace and dw_destroy.
+cudaError_t dw_pool_alloc(dw_ctx* c, size_t bytes, void** p, cudaStream_t s);
 
 // DW_OK when the calling thread's current device is the context's device; otherwise DW_EINVAL
 // with a message naming the entry point (kernels would mix memory of two devices).
@@ -495,8 +520,8 @@ void f64_to_dd(const double* x, dd* y, size_t n_real, cudaStream_t s);
 void dd_to_f64(const dd* x, double* y, size_t n_real, int add, cudaStream_t s);
 // make the context's double-float copies of the links and the clover term (once)
 int dw_make_dd(dw_ctx* c, cudaStream_t s);
-// out = D in on dd-form fields (FP64-class accuracy on the FP32 pipes)
-void dirac_full_dd(dw_ctx* c, const dd* in, dd* out, cudaStream_t s);
+// out = D in, or eta - D in with eta, for a dd-form field (FP64-class accuracy on the FP32 pipes)
+void dirac_full_dd(dw_ctx* c, const dd* in, const double* eta, double* out, cudaStream_t s);
 
 // dirac / sap entry points used by the solver ---------------------------------------
 // even-odd Schur operator (odd sites of out zero; uses the context's scratch field) and the

@@ -266,7 +266,13 @@ template void dirac_full<double>(dw_ctx*, const double*, double*, cudaStream_t);
 // sites): thread half q forms the spin-q component of every half-spinor projection, multiplies it
 // by the link and adds it to spin q and to the lower spin it feeds; the two halves exchange their
 // lower-spin partial sums through shared memory, and each applies rows 3q..3q+2 of both chiral
-// clover blocks.  Half the arithmetic and registers per thread of dirac_full_kernel<dd>.
+// clover blocks.  The double-float links are stored with all three rows: rebuilding the third one in
+// double-float arithmetic, in both halves, took a third of the operations, and the kernel uses a tenth of
+// the memory bandwidth.  The result leaves as FP64, D in or eta - D in.
+// Bound: FP32 issue and latency (20 warps per SM).  40x24x16x24, with the conversion of the input: 375 us;
+// unrolled over the directions 525 us, with the third row rebuilt and results and residual in passes of their
+// own 745 us; 4 CTAs per SM 3% more, 6 CTAs 10%.
+constexpr int DD_BLOCKS = 5;      // CTAs per SM
 // s + e = a b for double-float a, b, exact up to the product of the low parts (Dekker's product of
 // the leading parts by one FMA); s + e += a b with the leading part added by TwoSum and all errors
 // gathered in e (compensated dot product, Ogita, Rump and Oishi 2005)
@@ -283,17 +289,51 @@ DW_D void dd2_acc(float& s, float& e, dd a, dd b) {
   s = t;
   e = __fadd_rn(e, __fadd_rn(err, l));
 }
-// o = U h (DAG: U^+ h) in double-float precision, each output component a compensated sum of its
-// six real products (about 40% fewer FP32 operations than product-by-product double-float arithmetic)
-template <bool DAG>
-DW_D void su3_mul_dd2(const SU3<dd>& U, const cplx<dd>* h, cplx<dd>* o) {
+DW_D float flip(float x, uint32_t m) { return __uint_as_float(__float_as_uint(x) ^ m); }     // m: 0 or the sign bit
+DW_D dd flip(dd x, uint32_t m) { return {flip(x.hi, m), flip(x.lo, m)}; }
+
+// One hop of half q of a site, direction d = 2 mu + (1: backward), from the neighbour's spinor at P and the link
+// at Lk (unit planes of stride V): au += sign w, and the lower spin that w feeds, own (2 + q) or the other
+// one, += its image.  d is a run-time value: unrolled over the eight directions the kernel's code exceeds the
+// instruction caches and warps wait for instructions.  Multiplications by +-1 and +-i are sign flips
+// and exchanges of real and imaginary parts.
+//   v = e_mu-part of the lower spin:  mu 0: -psi_lo, 1: -i psi_lo, 2: (q ? +1 : -1) psi_lo, 3: (q ? +i : -i) psi_lo
+//   h = psi_q + S v, S = -1 forward, +1 backward;  w = U h (backward: U^+ h)
+//   image of w:                       mu 0: -w, 1: i w, 2: (q ? +1 : -1) w, 3: (q ? -i : +i) w;  times S
+DW_D void dd_half_hop(int d, const float4* __restrict__ Lk, const float4* __restrict__ P, size_t V, int q, bool wrap,
+                      cplx<dd>* au, cplx<dd>* own, cplx<dd>* oth) {
+  constexpr uint32_t SIGN = 0x80000000u;
+  const int mu = d >> 1;
+  const bool back = d & 1, imag = mu & 1, mine = mu == 0 || mu == 3;      // the lower spin involved: 2 + q or 3 - q
+  const int lo = mine ? 2 + q : 3 - q;
+  // S v: coefficient +-1 or +-i; i z = (-im, re)
+  const bool vneg = ((mu < 2) || !q) != !back;
+  const uint32_t vr = (vneg != imag) ? SIGN : 0u, vi = vneg ? SIGN : 0u;
+  cplx<dd> h[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    cplx<dd> u, l;
+    unpack_unit(__ldg(P + (size_t)(3 * q + c) * V), &u);
+    unpack_unit(__ldg(P + (size_t)(3 * lo + c) * V), &l);
+    const dd a = imag ? l.im : l.re, b = imag ? l.re : l.im;
+    h[c] = {u.re + flip(a, vr), u.im + flip(b, vi)};
+  }
+  // w = U h or U^+ h, each component a compensated sum of its six real products (about 40% fewer FP32
+  // operations than product-by-product double-float arithmetic)
+  const size_t sa = back ? V : 3 * V, sc = back ? 3 * V : V;               // element (a, c) or (c, a)
+  const uint32_t cj = back ? SIGN : 0u;
+  const uint32_t sg = wrap ? SIGN : 0u;
+  // the image: S (times the wrap sign) and +-1 or +-i
+  const bool wneg = (mu == 0 || (mu == 2 && !q) || (mu == 3 && q)) != !back;
+  const uint32_t wr = ((wneg != imag) ? SIGN : 0u) ^ sg, wi = (wneg ? SIGN : 0u) ^ sg;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     float sr, er, si, ei;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const cplx<dd> u = DAG ? U.m[c][a] : U.m[a][c];
-      const dd ui = DAG ? -u.im : u.im;               // conj(U)^T for the adjoint
+      cplx<dd> u;
+      unpack_unit(__ldg(Lk + a * sa + c * sc), &u);
+      const dd ui = flip(u.im, cj);
       if (c == 0) {
         dd2_first(sr, er, u.re, h[c].re);
         dd2_first(si, ei, u.re, h[c].im);
@@ -304,74 +344,61 @@ DW_D void su3_mul_dd2(const SU3<dd>& U, const cplx<dd>* h, cplx<dd>* o) {
       dd2_acc(sr, er, -ui, h[c].im);
       dd2_acc(si, ei, ui, h[c].re);
     }
-    o[a] = {dd_two_sum(sr, er), dd_two_sum(si, ei)};
+    const dd wre = dd_two_sum(sr, er), wim = dd_two_sum(si, ei);
+    au[a] += cplx<dd>{flip(wre, sg), flip(wim, sg)};
+    const cplx<dd> l = {flip(imag ? wim : wre, wr), flip(imag ? wre : wim, wi)};
+    if (mine) own[a] += l; else oth[a] += l;
   }
 }
 
-template <int MU, bool DAG>
-DW_D void dd_half_hop(const dd* __restrict__ links, const dd* __restrict__ in, size_t V, long long j,
-                      long long lk, int q, bool flip, cplx<dd>* au, cplx<dd>* al2, cplx<dd>* al3) {
-  // lower spin feeding / fed by component q: 2 + q for mu = 0, 3; 3 - q for mu = 1, 2
-  const int lo = (MU == 0 || MU == 3) ? 2 + q : 3 - q;
-  SU3<dd> U;
-  load_link(links, V, MU, lk, U);
-  cplx<dd> pu[3], pl[3];
-  const float4* P = reinterpret_cast<const float4*>(in);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    unpack_unit(__ldg(P + (size_t)(3 * q + c) * V + j), pu + c);
-    unpack_unit(__ldg(P + (size_t)(3 * lo + c) * V + j), pl + c);
-  }
-  // v_q = e_mu-part of the lower spins: mu 0: -psi_lo; 1: -i psi_lo; 2: (q ? +1 : -1) psi_lo;
-  // 3: (q ? +i : -i) psi_lo.  h = psi_q + S v_q with S = -1 forward (DAG = false), +1 backward.
-  // S = +1 (DAG) or -1, sg = -1 (flip: antiperiodic wrap) or +1: products with them are sign flips
-  cplx<dd> h[3], w[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    cplx<dd> v;
-    if (MU == 0) v = -pl[c];
-    else if (MU == 1) v = -ti(pl[c]);
-    else if (MU == 2) v = q ? pl[c] : -pl[c];
-    else v = q ? ti(pl[c]) : -ti(pl[c]);
-    h[c] = DAG ? pu[c] + v : pu[c] - v;
-  }
-  su3_mul_dd2<DAG>(U, h, w);
-  // the lower-spin image of w_q: mu 0: -w; 1: i w; 2: (q ? +w : -w); 3: (q ? -i w : i w)
-  const bool neg_lower = (!DAG) != flip;               // S sg = -1
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    au[c] += flip ? -w[c] : w[c];
-    cplx<dd> l;
-    if (MU == 0) l = -w[c];
-    else if (MU == 1) l = ti(w[c]);
-    else if (MU == 2) l = q ? w[c] : -w[c];
-    else l = q ? -ti(w[c]) : ti(w[c]);
-    const cplx<dd> add = neg_lower ? -l : l;
-    if (lo == 2) al2[c] += add; else al3[c] += add;
-  }
-}
-
-// rows r0..r0+2 of one packed Hermitian 6x6 chiral block times x (6 components)
+// rows R0..R0+2 of one packed Hermitian 6x6 chiral block (18 slots at blk, stride V) times x (6
+// components): the off-diagonal products of a component as one compensated sum, whose error is that of
+// these smaller terms, then the diagonal one in double-float arithmetic
 template <int R0>
-DW_D void herm6_rows(const cplx<dd>* s, const cplx<dd>* x, cplx<dd>* y) {
-  const dd d[6] = {s[0].re, s[0].im, s[1].re, s[1].im, s[2].re, s[2].im};
+DW_D void herm6_rows(const float4* __restrict__ blk, size_t V, const cplx<dd>* x, cplx<dd>* y) {
+  float sr[3], er[3], si[3], ei[3];
 #pragma unroll
-  for (int r = 0; r < 3; ++r) y[r] = d[R0 + r] * x[R0 + r];
+  for (int r = 0; r < 3; ++r) sr[r] = er[r] = si[r] = ei[r] = 0.f;
   int k = 3;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
 #pragma unroll
     for (int j = i + 1; j < 6; ++j) {
-      if (i >= R0 && i < R0 + 3) y[i - R0] += s[k] * x[j];
-      if (j >= R0 && j < R0 + 3) y[j - R0] += cmulc(s[k], x[i]);
+      const bool ri = i >= R0 && i < R0 + 3, rj = j >= R0 && j < R0 + 3;
+      if (ri || rj) {
+        cplx<dd> m;
+        unpack_unit(__ldg(blk + (size_t)k * V), &m);
+        if (ri) {                                        // y_i += m x_j
+          const int r = i - R0;
+          dd2_acc(sr[r], er[r], m.re, x[j].re);
+          dd2_acc(si[r], ei[r], m.re, x[j].im);
+          dd2_acc(sr[r], er[r], -m.im, x[j].im);
+          dd2_acc(si[r], ei[r], m.im, x[j].re);
+        }
+        if (rj) {                                        // y_j += conj(m) x_i
+          const int r = j - R0;
+          dd2_acc(sr[r], er[r], m.re, x[i].re);
+          dd2_acc(si[r], ei[r], m.re, x[i].im);
+          dd2_acc(sr[r], er[r], m.im, x[i].im);
+          dd2_acc(si[r], ei[r], -m.im, x[i].re);
+        }
+      }
       ++k;
     }
   }
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    cplx<dd> d2;
+    unpack_unit(__ldg(blk + (size_t)((R0 + r) / 2) * V), &d2);
+    const dd d = (R0 + r) % 2 ? d2.im : d2.re;
+    y[r] = {dd_two_sum(sr[r], er[r]) + d * x[R0 + r].re, dd_two_sum(si[r], ei[r]) + d * x[R0 + r].im};
+  }
 }
 
-__global__ void __launch_bounds__(128) dirac_dd_split_kernel(Geom g, const dd* __restrict__ links,
-                                                             const dd* __restrict__ clov, const dd* __restrict__ in,
-                                                             dd* __restrict__ out) {
+__global__ void __launch_bounds__(128, DD_BLOCKS) dirac_dd_split_kernel(Geom g, const float4* __restrict__ links,
+                                                             const float4* __restrict__ clov,
+                                                             const dd* __restrict__ in, const double2* eta,
+                                                             double2* out) {
   __shared__ cplx<dd> xch[2][3][64];          // lower-spin partials handed to the other half
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int q = w & 1, grp = w >> 1;           // warp-uniform half
@@ -379,82 +406,71 @@ __global__ void __launch_bounds__(128) dirac_dd_split_kernel(Geom g, const dd* _
   const long long i = (long long)blockIdx.x * 64 + sl;
   const bool valid = i < g.V;
   const size_t V = g.V;
-  cplx<dd> au[3], a2[3], a3[3];
+  cplx<dd> au[3], al[3], ao[3];                // upper spin q, lower spins 2 + q and 3 - q
 #pragma unroll
-  for (int c = 0; c < 3; ++c) { au[c] = {dd(0), dd(0)}; a2[c] = au[c]; a3[c] = au[c]; }
+  for (int c = 0; c < 3; ++c) { au[c] = {dd(0), dd(0)}; al[c] = au[c]; ao[c] = au[c]; }
   if (valid) {
     const SiteRef s = decode(g, i);
-    bool cr;
-#define DD_DIR(MU)                                                                        \
-    {                                                                                     \
-      long long j = neighbour(g, s, 2 * MU, &cr);                                         \
-      bool flip = time_wrap(g, s, 2 * MU);                                                \
-      dd_half_hop<MU, false>(links, in, V, j, i, q, flip, au, a2, a3);                    \
-      j = neighbour(g, s, 2 * MU + 1, &cr);                                               \
-      flip = time_wrap(g, s, 2 * MU + 1);                                                 \
-      dd_half_hop<MU, true>(links, in, V, j, j, q, flip, au, a2, a3);                     \
+#pragma unroll 1
+    for (int d = 0; d < 8; ++d) {
+      bool cr;
+      const long long j = neighbour(g, s, d, &cr);
+      dd_half_hop(d, links + (size_t)((d >> 1) * 9) * V + (d & 1 ? j : i), reinterpret_cast<const float4*>(in) + j, V, q,
+                  time_wrap(g, s, d), au, al, ao);
     }
-    DD_DIR(0) DD_DIR(1) DD_DIR(2) DD_DIR(3)
-#undef DD_DIR
   }
-  // half q keeps lower spin 2 + q: hand the other lower spin to the partner half
+  // hand the other lower spin to the partner half
 #pragma unroll
-  for (int c = 0; c < 3; ++c) xch[q][c][sl] = q ? a2[c] : a3[c];
+  for (int c = 0; c < 3; ++c) xch[q][c][sl] = ao[c];
   __syncthreads();
   if (!valid) return;
-  cplx<dd> al[3];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) al[c] = (q ? a3[c] : a2[c]) + xch[1 - q][c][sl];
+  for (int c = 0; c < 3; ++c) al[c] += xch[1 - q][c][sl];
   // clover: rows 3q..3q+2 of both chiral blocks (block 0: spins 0, 1; block 1: spins 2, 3)
-  cplx<dd> x[6], sblk[18], y0[3], y1[3];
+  cplx<dd> x[6], y[3];
   const float4* P = reinterpret_cast<const float4*>(in);
-#pragma unroll
-  for (int k = 0; k < 6; ++k) unpack_unit(__ldg(P + (size_t)k * V + i), x + k);
-  load_site<dd, 18>(clov, V, i, sblk);
-  if (q) herm6_rows<3>(sblk, x, y0); else herm6_rows<0>(sblk, x, y0);
-#pragma unroll
-  for (int k = 0; k < 6; ++k) unpack_unit(__ldg(P + (size_t)(6 + k) * V + i), x + k);
-  load_site<dd, 18>(clov + 36 * V, V, i, sblk);
-  if (q) herm6_rows<3>(sblk, x, y1); else herm6_rows<0>(sblk, x, y1);
-  // out spin q (block 0 rows 3q..) and spin 2 + q (block 1 rows 3q..)
-  float4* O = reinterpret_cast<float4*>(out);
   const dd hf = dd(0.5f);
+  // out spin q (block 0 rows 3q..) and spin 2 + q (block 1 rows 3q..)
+#pragma unroll 1
+  for (int blk = 0; blk < 2; ++blk) {
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const cplx<dd> u = y0[c] - hf * au[c];
-    const cplx<dd> l = y1[c] - hf * al[c];
-    O[(size_t)(3 * q + c) * V + i] = pack_unit(&u);
-    O[(size_t)(3 * (2 + q) + c) * V + i] = pack_unit(&l);
+    for (int k = 0; k < 6; ++k) unpack_unit(__ldg(P + (size_t)(6 * blk + k) * V + i), x + k);
+    const float4* cb = clov + (size_t)(18 * blk) * V + i;
+    if (q) herm6_rows<3>(cb, V, x, y); else herm6_rows<0>(cb, V, x, y);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const cplx<dd> u = y[c] - hf * (blk ? al[c] : au[c]);
+      const size_t o = (size_t)(3 * (2 * blk + q) + c) * V + i;
+      double2 r = make_double2(widen(u.re.hi) + widen(u.re.lo), widen(u.im.hi) + widen(u.im.lo));
+      if (eta) {
+        const double2 e = eta[o];
+        r = make_double2(e.x - r.x, e.y - r.y);
+      }
+      out[o] = r;
+    }
   }
 }
 
-void dirac_full_dd(dw_ctx* c, const dd* in, dd* out, cudaStream_t st) {
-  const char* e = getenv("DW_DD_SPLIT");
-  if (e && e[0] == '0') {
-    unsigned blocks = (unsigned)((c->V + 127) / 128);
-    dirac_full_kernel<dd><<<blocks, 128, 0, st>>>(c->g, (const dd*)c->links_dd, (const dd*)c->clov_dd, in, out);
-  } else {
-    unsigned blocks = (unsigned)((c->V + 63) / 64);
-    dirac_dd_split_kernel<<<blocks, 128, 0, st>>>(c->g, (const dd*)c->links_dd, (const dd*)c->clov_dd, in, out);
-  }
+void dirac_full_dd(dw_ctx* c, const dd* in, const double* eta, double* out, cudaStream_t st) {
+  unsigned blocks = (unsigned)((c->V + 63) / 64);
+  dirac_dd_split_kernel<<<blocks, 128, 0, st>>>(c->g, (const float4*)c->links_dd, (const float4*)c->clov_dd, in,
+                                                (const double2*)eta, (double2*)out);
   dw_note_launch();
 }
 
-// FP64 fields through double-float arithmetic: convert, apply, convert back (nrhs fields)
+// FP64 fields through double-float arithmetic (nrhs fields, one converted at a time; the converted field comes
+// from the context's own memory pool, which keeps it for the next call of whatever stream)
 static int dirac_full_f64x(dw_ctx* c, const double* in, double* out, int nrhs, cudaStream_t st) {
   int rc = dw_make_dd(c, st);
   if (rc) return rc;
   const size_t n = (size_t)c->V * 24;
-  dd *a = nullptr, *b = nullptr;
-  DW_CUDA(cudaMallocAsync(&a, n * sizeof(dd), st));
-  DW_CUDA(cudaMallocAsync(&b, n * sizeof(dd), st));
+  dd* a = nullptr;
+  DW_CUDA(dw_pool_alloc(c, n * sizeof(dd), (void**)&a, st));
   for (int r = 0; r < nrhs; ++r) {
     f64_to_dd(in + r * n, a, n, st);
-    dirac_full_dd(c, a, b, st);
-    dd_to_f64(b, out + r * n, n, 0, st);
+    dirac_full_dd(c, a, nullptr, out + r * n, st);
   }
   DW_CUDA(cudaFreeAsync(a, st));
-  DW_CUDA(cudaFreeAsync(b, st));
   return DW_OK;
 }
 

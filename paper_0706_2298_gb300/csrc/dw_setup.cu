@@ -100,6 +100,21 @@ __device__ void leaf(const SU3<double>& A, const SU3<double>& B, const SU3<doubl
     for (int b = 0; b < 3; ++b) Q.m[a][b] += t1.m[a][b];
 }
 
+// row 2 = conj(row 0 x row 1) of the FP64 links
+__global__ void link_row2_kernel(long long V, double2* links) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t >= 4 * V) return;
+  const long long mu = t / V, i = t % V;
+  double2* u = links + mu * 9 * V + i;
+  cplx<double> r[6];
+  for (int k = 0; k < 6; ++k) unpack_unit(u[k * V], r + k);
+  for (int j = 0; j < 3; ++j) {
+    const int a = (j + 1) % 3, b = (j + 2) % 3;
+    const cplx<double> x = conjg(r[a] * r[3 + b] - r[b] * r[3 + a]);
+    u[(6 + j) * V] = pack_unit(&x);
+  }
+}
+
 __global__ void clover_build_kernel(Geom g, const double* __restrict__ links, SigmaTable sig, double diag,
                                     double csw, double* cl64, double* ci64, float* cl32, float* ci32,
                                     int* bad) {
@@ -269,6 +284,7 @@ static void free_ctx(dw_ctx* c) {
   sap_graphs_free(c);
   for (auto& a : c->ws_solve) a.release();
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
+  if (c->pool) cudaMemPoolDestroy(c->pool);
   void* ptrs[] = {c->d_canon_of, c->d_nbtab, c->d_blk_nb, c->d_blk_x0, c->d_loc, c->d_colour_list,
                   c->links[0], c->links[1], c->clov[0], c->clov[1], c->clovinv[0], c->clovinv[1],
                   c->sap_r[0], c->sap_r[1], c->sap_d[0], c->sap_d[1], c->d_red, c->d_count,
@@ -289,6 +305,7 @@ extern "C" int dw_release_workspace(dw_ctx* c) {
   for (auto& a : c->ws_solve) a.release();
   if (c->links_dd) { cudaFree(c->links_dd); c->links_dd = nullptr; }
   if (c->clov_dd) { cudaFree(c->clov_dd); c->clov_dd = nullptr; }
+  if (c->pool) { cudaMemPoolDestroy(c->pool); c->pool = nullptr; }
   return DW_OK;
 }
 
@@ -457,7 +474,7 @@ extern "C" int dw_create(const dw_params* p, const double* links_host, dw_ctx** 
       (rc = up((void**)&c->d_blk_x0, blk_x0.data(), blk_x0.size() * sizeof(int))) ||
       (rc = up((void**)&c->d_loc, loc.data(), loc.size() * sizeof(uchar4))) ||
       (rc = up((void**)&c->d_colour_list, colour_list.data(), colour_list.size() * sizeof(int))) ||
-      (rc = up(&c->links[DW_F64], l64.data(), l64.size())) ||
+      (rc = up(&c->links[DW_F64], nullptr, (size_t)V * 4 * 18 * 8)) ||
       (rc = up(&c->links[DW_F32], l32.data(), l32.size())) ||
       (rc = up(&c->clov[DW_F64], nullptr, (size_t)V * 72 * 8)) ||
       (rc = up(&c->clov[DW_F32], nullptr, (size_t)V * 72 * 4)) ||
@@ -468,6 +485,11 @@ extern "C" int dw_create(const dw_params* p, const double* links_host, dw_ctx** 
     free_ctx(c);
     return rc;
   }
+  // FP64 links: rows 0 and 1 of a direction, then its row 2
+  for (int mu = 0; mu < 4; ++mu)
+    cudaMemcpy((double*)c->links[DW_F64] + (size_t)mu * 18 * V, l64.data() + (size_t)mu * 12 * V * 8,
+               (size_t)12 * V * 8, cudaMemcpyHostToDevice);
+  link_row2_kernel<<<(unsigned)((4 * V + 255) / 256), 256>>>(V, (double2*)c->links[DW_F64]); dw_note_launch();
   cudaMemset(c->d_count, 0, 64 * sizeof(unsigned));
   if (cudaMallocHost((void**)&c->h_red, 1 << 16) != cudaSuccess) {
     free_ctx(c);

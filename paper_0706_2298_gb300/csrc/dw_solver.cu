@@ -112,7 +112,7 @@ struct Work {
   std::vector<T*> xi, chi;
   T *rho = nullptr, *w = nullptr, *t1 = nullptr, *lc = nullptr, *lv = nullptr;
   double *eta = nullptr, *psi = nullptr, *r64 = nullptr, *t64 = nullptr, *c64 = nullptr, *v64 = nullptr;
-  dd *dda = nullptr, *ddb = nullptr;     // double-float fields of the mixed restarts
+  dd* dda = nullptr;                     // double-float field of the mixed restarts
   WsArena& arena;
   explicit Work(WsArena& a) : arena(a) { arena.rewind(); }
   int alloc(size_t bytes, void** p) {
@@ -169,21 +169,18 @@ int solve_one(dw_ctx* c, dfl_ctx* d, const sol_params* p, const double* eta_cano
     return DW_OK;
   }
   if (p->mixed) {      // restart steps in double-float arithmetic on the FP32 pipes
-    if ((rc = dw_make_dd(c, s)) || (rc = W.alloc(V * 24 * sizeof(dd), (void**)&W.dda)) ||
-        (rc = W.alloc(V * 24 * sizeof(dd), (void**)&W.ddb)))
-      return rc;
+    if ((rc = dw_make_dd(c, s)) || (rc = W.alloc(V * 24 * sizeof(dd), (void**)&W.dda))) return rc;
   }
   auto residual64 = [&]() -> int {   // r64 = eta - D psi, returns via h[2] = |r|^2
     tm.begin(PH_RESTART);
     if (p->mixed) {
       f64_to_dd(W.psi, W.dda, V * 24, s);
-      dirac_full_dd(c, W.dda, W.ddb, s);
-      dd_to_f64(W.ddb, W.t64, V * 24, 0, s);
+      dirac_full_dd(c, W.dda, W.eta, W.r64, s);
     } else {
       dirac_full<double>(c, W.psi, W.t64, s);
+      DW_CUDA(cudaMemcpyAsync(W.r64, W.eta, fb64, cudaMemcpyDeviceToDevice, s));
+      blas_axpy<double>(W.t64, W.r64, -1.0, 0.0, n, s);
     }
-    DW_CUDA(cudaMemcpyAsync(W.r64, W.eta, fb64, cudaMemcpyDeviceToDevice, s));
-    blas_axpy<double>(W.t64, W.r64, -1.0, 0.0, n, s);
     blas_dot<double>(c, W.r64, W.r64, n, dres, s);
     tm.end();
     return read_host(c, dres, 3, h, s);
@@ -372,19 +369,14 @@ int solve_batch_f32(dw_ctx* c, dfl_ctx* d, const sol_params* p, int nrhs, const 
   std::vector<double> lrr(nrhs);
   if ((rc = norms64(W.eta, en))) return rc;
   for (int r = 0; r < nrhs; ++r) conv[r] = en[r] == 0.0;
-  dd *dda = nullptr, *ddb = nullptr;
-  if ((rc = dw_make_dd(c, s)) || (rc = W.alloc(fs * sizeof(dd), (void**)&dda)) ||
-      (rc = W.alloc(fs * sizeof(dd), (void**)&ddb)))
-    return rc;
+  dd* dda = nullptr;
+  if ((rc = dw_make_dd(c, s)) || (rc = W.alloc(fs * sizeof(dd), (void**)&dda))) return rc;
   auto residual64 = [&]() -> int {   // restart residuals in double-float arithmetic
     tm.begin(PH_RESTART);
     for (int r = 0; r < nrhs; ++r) {
       f64_to_dd(F64(W.psi, r), dda, fs, s);
-      dirac_full_dd(c, dda, ddb, s);
-      dd_to_f64(ddb, F64(W.t64, r), fs, 0, s);
+      dirac_full_dd(c, dda, F64(W.eta, r), F64(W.r64, r), s);
     }
-    DW_CUDA(cudaMemcpyAsync(W.r64, W.eta, fb64, cudaMemcpyDeviceToDevice, s));
-    blas_axpy<double>(W.t64, W.r64, -1.0, 0.0, n * nrhs, s);   // the batch's fields are contiguous
     tm.end();
     return norms64(W.r64, rn);
   };
