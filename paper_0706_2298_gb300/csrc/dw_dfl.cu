@@ -337,63 +337,71 @@ struct WarpHalve {
   }
 };
 
-// c[L][k] = (phi^L_k, psi), Ns known at compile time: CTA per deflation block, per-thread
-// partial sums in the working precision, CTA sum by warp halving + shared memory.
+// c[L][k] = (phi^L_k, psi), Ns known at compile time: CTA per deflation block, four groups of 128
+// threads, each for a quarter of the basis vectors and all sites of the block; per-thread partial sums, CTA
+// sum by warp halving + shared memory.
+// Bound: HBM (the basis).  A thread with all Ns vectors needs 2 Ns accumulators and 32 KB of unrolled code, and
+// 16 warps per SM did not keep enough loads in flight: 40x24x16x24, Ns = 20: 97 -> 79 us (4.9 TB/s); two groups 91 us.
+constexpr int RK_G = 4;
 template <typename T, int NS>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2) restrict_ns_kernel(Geom g, const int* __restrict__ sub, int nsub,
+__global__ void __launch_bounds__(128 * RK_G, sizeof(T) == 4 ? 2 : 1) restrict_ns_kernel(Geom g, const int* __restrict__ sub, int nsub,
                                                              const double* b64, const uint4* b16,
                                                              const T* __restrict__ psi0, T* __restrict__ c0,
                                                              int nrhs, size_t fstride, size_t cstride) {
-  using WH = WarpHalve<T, 2 * NS, 16>;
+  static_assert(NS % RK_G == 0, "the groups share the basis vectors evenly");
+  constexpr int KP = NS / RK_G;
+  using WH = WarpHalve<T, 2 * KP, 16>;
   constexpr int MF = WH::final_m();
-  __shared__ T sh[4][2 * NS];
+  __shared__ T sh[4 * RK_G][2 * KP];
   const int L = blockIdx.x;
   const size_t V = g.V;
   const int nsite = nsub * g.svol;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int grp = threadIdx.x >> 7, tl = threadIdx.x & 127, k0 = grp * KP;
   for (int rhs = 0; rhs < nrhs; ++rhs) {
     const T* psi = psi0 + (size_t)rhs * fstride;
     T* c = c0 + (size_t)rhs * cstride;
-    T acc[2 * NS];
+    cplx<T> acc[KP];
 #pragma unroll
-    for (int k = 0; k < 2 * NS; ++k) acc[k] = T(0);
-    for (int t = threadIdx.x; t < nsite; t += blockDim.x) {
+    for (int k = 0; k < KP; ++k) acc[k] = {T(0), T(0)};
+    for (int t = tl; t < nsite; t += 128) {
       const long long i = dfl_site(g, sub, nsub, L, t);
       cplx<T> p[12];
       load_site<T, 12>(psi, V, i, p);
 #pragma unroll
-      for (int k = 0; k < NS; ++k) {
-        cplx<T> f[12];
-        load_basis<T>(b64, b16, V, k, i, f);
-        T re = 0, im = 0;
+      for (int k = 0; k < KP; ++k) {
+        cplx<T> f[12], s = {T(0), T(0)};
+        load_basis<T>(b64, b16, V, k0 + k, i, f);
 #pragma unroll
-        for (int j = 0; j < 12; ++j) {
-          re += f[j].re * p[j].re + f[j].im * p[j].im;
-          im += f[j].re * p[j].im - f[j].im * p[j].re;
-        }
-        acc[2 * k] += re;
-        acc[2 * k + 1] += im;
+        for (int j = 0; j < 12; ++j) cmacc(s, f[j], p[j]);
+        acc[k] += s;
       }
     }
+    T x[2 * KP];
+#pragma unroll
+    for (int k = 0; k < KP; ++k) { x[2 * k] = acc[k].re; x[2 * k + 1] = acc[k].im; }
     int base = 0;
-    WH::run(acc, lane, base);
+    WH::run(x, lane, base);
     // lanes holding the same index block hold equal sums; all of them store
 #pragma unroll
-    for (int m = 0; m < MF; ++m) sh[w][base + m] = acc[m];
+    for (int m = 0; m < MF; ++m) sh[w][base + m] = x[m];
     __syncthreads();
-    if (threadIdx.x < 2 * NS) {
-      T y = sh[0][threadIdx.x];
+    if (tl < 2 * KP) {                 // warps 4 grp .. 4 grp + 3 hold group grp's sums
+      T y = sh[4 * grp][tl];
 #pragma unroll
-      for (int q = 1; q < 4; ++q) y += sh[q][threadIdx.x];
-      c[(size_t)L * 2 * NS + threadIdx.x] = y;
+      for (int q = 1; q < 4; ++q) y += sh[4 * grp + q][tl];
+      c[(size_t)L * 2 * NS + 2 * k0 + tl] = y;
     }
     __syncthreads();
   }
 }
 
 // psi = mode 0: Phi c ; 1: psi + Phi c ; 2: psi - Phi c
-template <typename T>
-__global__ void __launch_bounds__(128) prolong_kernel(Geom g, const int* __restrict__ sap2dfl, int Ns,
+// A thread per site; CTAs of BLOCK threads.  FP32: 256 threads (4 KB pieces of the basis' unit planes) and 24
+// warps per SM: 78 us at 40x24x16x24, Ns = 20 (5.0 TB/s), 34 us at 24x16^3, Ns = 32; 128 threads 87 and 49 us,
+// but they fill the chip on lattices below 2 x 256 sites per SM (16^4, Ns = 12: 8.7 against 10.6 us).
+template <typename T, int BLOCK>
+__global__ void __launch_bounds__(BLOCK, sizeof(T) != 4 ? 1 : BLOCK == 256 ? 3 : 5) prolong_kernel(Geom g, const int* __restrict__ sap2dfl, int Ns,
                                                       const double* b64, const uint4* b16,
                                                       const T* __restrict__ c0, T* psi0, int mode, int nrhs,
                                                       size_t fstride, size_t cstride) {
@@ -412,12 +420,13 @@ __global__ void __launch_bounds__(128) prolong_kernel(Geom g, const int* __restr
     load_site_rw<T, 12>(psi, V, i, out);
   }
   const cplx<T>* cc = reinterpret_cast<const cplx<T>*>(c) + (size_t)L * Ns;
+#pragma unroll 4
   for (int k = 0; k < Ns; ++k) {
     cplx<T> ck = cc[k];
     if (mode == 2) ck = -ck;
     load_basis<T>(b64, b16, V, k, i, f);
 #pragma unroll
-    for (int j = 0; j < 12; ++j) out[j] += ck * f[j];
+    for (int j = 0; j < 12; ++j) cmac(out[j], ck, f[j]);
   }
   store_site<T, 12>(psi, V, i, out);
   }
@@ -2076,9 +2085,9 @@ static bool launch_restrict_ns(dfl_ctx* d, const T* psi, T* c, int nrhs, cudaStr
   if constexpr (NS == 0 || !std::is_same<T, float>::value) {
     return false;
   } else {
-    restrict_ns_kernel<T, NS><<<d->Nb, 128, 0, s>>>(d->c->g, d->d_sub, d->nsub, d->basis16 ? nullptr : d->basis64,
-                                                    d->basis16, psi, c, nrhs, (size_t)d->c->V * 24,
-                                                    (size_t)d->N * 2);
+    restrict_ns_kernel<T, NS><<<d->Nb, 128 * RK_G, 0, s>>>(d->c->g, d->d_sub, d->nsub,
+                                                           d->basis16 ? nullptr : d->basis64, d->basis16, psi, c, nrhs,
+                                                           (size_t)d->c->V * 24, (size_t)d->N * 2);
     return true;
   }
 }
@@ -2096,10 +2105,15 @@ static int restrict_t(dfl_ctx* d, const T* psi, T* c, cudaStream_t s, int nrhs =
 }
 template <typename T>
 static int prolong_t(dfl_ctx* d, const T* c, T* psi, int mode, cudaStream_t s, int nrhs = 1) {
-  unsigned blocks = (unsigned)((d->c->V + 127) / 128);
-  prolong_kernel<T><<<blocks, 128, 0, s>>>(d->c->g, d->d_sap2dfl, d->Ns, d->basis16 ? nullptr : d->basis64,
-                                            d->basis16, c, psi, mode, nrhs, (size_t)d->c->V * 24,
-                                            (size_t)d->N * 2); dw_note_launch();
+  const size_t V = d->c->V;
+  const double* b64 = d->basis16 ? nullptr : d->basis64;
+  if (sizeof(T) == 4 && V / 256 >= 2 * (size_t)d->c->sms)
+    prolong_kernel<T, 256><<<(unsigned)((V + 255) / 256), 256, 0, s>>>(d->c->g, d->d_sap2dfl, d->Ns, b64, d->basis16, c,
+                                                                       psi, mode, nrhs, V * 24, (size_t)d->N * 2);
+  else
+    prolong_kernel<T, 128><<<(unsigned)((V + 127) / 128), 128, 0, s>>>(d->c->g, d->d_sap2dfl, d->Ns, b64, d->basis16, c,
+                                                                       psi, mode, nrhs, V * 24, (size_t)d->N * 2);
+  dw_note_launch();
   return DW_OK;
 }
 // s + e += f x for an FP32 number f and a double-float x: the product split exactly into
@@ -2180,7 +2194,8 @@ __global__ void __launch_bounds__(128 * KG) restrict_dd_bf16_kernel(Geom g, cons
 
 // psi = Phi c (the prolongation) for a double-float c and the BF16 basis: every output component a
 // compensated sum (dot2_acc) of its 2 Ns products of an exact FP32 basis entry with a double-float
-// coefficient; one thread per site.
+// coefficient; one thread per site.  The loop over the vectors stays rolled: unrolled by four it has 30 KB of
+// code (40x24x16x24: 274 us with the conversions, 242 rolled).
 template <int NS>
 __global__ void __launch_bounds__(128) prolong_dd_bf16_kernel(Geom g, const int* __restrict__ sap2dfl,
                                                               const uint4* __restrict__ b16,
@@ -2193,7 +2208,7 @@ __global__ void __launch_bounds__(128) prolong_dd_bf16_kernel(Geom g, const int*
   float sa[24], ea[24];
 #pragma unroll
   for (int m = 0; m < 24; ++m) sa[m] = ea[m] = 0.f;
-#pragma unroll 4
+#pragma unroll 1
   for (int k = 0; k < NS; ++k) {
     const cplx<dd> ck = cc[k];
     cplx<float> f[12];
@@ -2226,8 +2241,9 @@ static bool launch_restrict_dd(dfl_ctx* d, const dd* psi, dd* c, cudaStream_t s)
       restrict_dd_bf16_kernel<NS, (NS % 4 == 0 ? 4 : 2)><<<d->Nb, 128 * (NS % 4 == 0 ? 4 : 2), 0, s>>>(
           d->c->g, d->d_sub, d->nsub, d->basis16, psi, c, 1, (size_t)d->c->V * 24, (size_t)d->N * 2);
     else
-      restrict_ns_kernel<dd, NS><<<d->Nb, 128, 0, s>>>(d->c->g, d->d_sub, d->nsub, d->basis16 ? nullptr : d->basis64,
-                                                       d->basis16, psi, c, 1, (size_t)d->c->V * 24, (size_t)d->N * 2);
+      restrict_ns_kernel<dd, NS><<<d->Nb, 128 * RK_G, 0, s>>>(d->c->g, d->d_sub, d->nsub,
+                                                              d->basis16 ? nullptr : d->basis64, d->basis16, psi, c, 1,
+                                                              (size_t)d->c->V * 24, (size_t)d->N * 2);
     return true;
   }
 }
@@ -2268,7 +2284,7 @@ int dfl_prolong_f64x(dfl_ctx* d, const double* c, double* psi, int add, cudaStre
   bool done = false;
   if (d->basis16 && !dd_dot2_disabled()) NS_DISPATCH_FEW(d->Ns, (done = launch_prolong_dd<NSV>(d, blocks, s)));
   if (!done)
-    prolong_kernel<dd><<<blocks, 128, 0, s>>>(d->c->g, d->d_sap2dfl, d->Ns, d->basis16 ? nullptr : d->basis64,
+    prolong_kernel<dd, 128><<<blocks, 128, 0, s>>>(d->c->g, d->d_sap2dfl, d->Ns, d->basis16 ? nullptr : d->basis64,
                                               d->basis16, d->ddl, d->ddf, 0, 1, (size_t)d->c->V * 24,
                                               (size_t)d->N * 2);
   dw_note_launch();
