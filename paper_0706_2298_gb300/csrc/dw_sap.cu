@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(SHV) sap_block_kernel(Geom g, const T* __restr
 // While the odd sites apply A_oo^{-1}, the even ones apply A_ee.
 // Bound: instruction issue and latency (16 warps per SM at 128 registers and 98 KB, issue slots 57% busy);
 // the rest is the two parities waiting for each other and tensor-memory loads.  48x24^3 on 4^4 blocks, 4
-// cycles of 4 steps: 1.44 ms (22 TFLOP/s); links in shared memory and the whole clover term in tensor
+// cycles of 4 steps: 1.42 ms (22 TFLOP/s); links in shared memory and the whole clover term in tensor
 // memory 1.60 ms; pulling both hop terms from shared memory with one thread per (site pair, spin) 1.78 ms.
 template <int SHV>
 struct SapCfg {
@@ -265,19 +265,21 @@ DW_D void tm_st2(uint32_t a, const float* v) {
                "r"(__float_as_uint(v[1])) : "memory");
 }
 DW_D void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// 18 consecutive columns (the wait is part of the statement: the registers are valid after it)
+// 18 consecutive columns; the registers are valid after tm_wait18, which every use of them depends on
 DW_D void tm_ld18(uint32_t a, float* v) {
-  uint32_t r[18];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%18];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%16,%17}, [%19];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17])
-      : "r"(a), "r"(a + 16) : "memory");
-#pragma unroll
-  for (int k = 0; k < 18; ++k) v[k] = __uint_as_float(r[k]);
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%16,%17}, [%19];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]), "=f"(v[16]),
+        "=f"(v[17])
+      : "r"(a), "r"(a + 16));
+}
+DW_D void tm_wait18(float* v) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
+                 "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]),
+                 "+f"(v[16]), "+f"(v[17]));
 }
 
 // CTA barriers of a subset: wait for, or only announce, the arrival of n threads at barrier id
@@ -335,7 +337,8 @@ struct SapBlock {
       tm_wait_st();
     }
   }
-  DW_D void link(int mu, SU3<float>& U) const {      // whole warps only (tensor memory)
+  // whole warps only (tensor memory); U may be used after link_wait
+  DW_D void link(int mu, SU3<float>& U) const {
     cplx<float>* m = &U.m[0][0];
     if constexpr (Cfg::TM) {
       tm_ld18(tm + mu * 18, &m[0].re);
@@ -346,12 +349,17 @@ struct SapBlock {
       m[8] = {l.x, l.y};
     }
   }
+  DW_D void link_wait(SU3<float>& U) const {
+    if constexpr (Cfg::TM) tm_wait18(&U.m[0][0].re);
+  }
   // y = A_oo^{-1} x (odd) or A_ee x (even)
   DW_D void clover(size_t V, long long i, const cplx<float>* x, cplx<float>* y) const {
     cplx<float> s[18];
     if constexpr (Cfg::TM) {
       tm_ld18(tm + 72, &s[0].re);
       tm_ld18(tm + 90, &s[9].re);
+      tm_wait18(&s[0].re);
+      tm_wait18(&s[9].re);
       herm6_mul(s, x, y);
 #pragma unroll
       for (int k = 0; k < 9; ++k) unpack_unit(fix4[k * NS + t], s + 2 * k);
@@ -411,25 +419,29 @@ DW_D void add_half(const cplx<float>* w, cplx<float>* acc) {
 template <int MU, int SHV>
 DW_D void sap_forward(const SapBlock<SHV>& sb, const SapNb& nb, cplx<float>* acc) {
   SU3<float> U;
+  cplx<float> p[12], w[6];
   sb.link(MU, U);
+  sb.get(sb.vec, SHV, nb.at(2 * MU), p);       // some site of the block where the hop leaves it
+  sb.link_wait(U);
   if (nb.in(2 * MU)) {
-    cplx<float> p[12], w[6];
-    sb.get(sb.vec, SHV, nb.at(2 * MU), p);
     half_spinor<MU, -1, false>(p, U, w);
     add_half<MU, -1>(w, acc);
   }
 }
-// half-spinors U_mu(y)^+ (1 + gamma_mu) psi(y) of the owner's spinor
+// half-spinors U_mu(y)^+ (1 + gamma_mu) psi(y) of the owner's spinor; U is the link of direction MU on its way,
+// and is left as that of MU + 1
 template <int MU, int SHV>
-DW_D void sap_push(const SapBlock<SHV>& sb, const SapNb& nb, int h, const cplx<float>* psi) {
-  SU3<float> U;
-  sb.link(MU, U);
+DW_D void sap_push(const SapBlock<SHV>& sb, const SapNb& nb, int h, const cplx<float>* psi, SU3<float>& U) {
+  sb.link_wait(U);
+  SU3<float> next;
+  if (MU < 3) sb.link(MU + 1, next);
   if (nb.in(2 * MU)) {
     cplx<float> w[6];
     half_spinor<MU, +1, true>(psi, U, w);
 #pragma unroll
     for (int k = 0; k < 3; ++k) sb.half[(MU * 3 + k) * SHV + h] = pack_unit(w + 2 * k);
   }
+  if (MU < 3) U = next;
 }
 // acc += the backward term of direction mu, from the half-spinor of x - mu
 template <int MU, int SHV>
@@ -617,10 +629,12 @@ __global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
         sap_forward<2>(sb, nb, a);
         sap_forward<3>(sb, nb, a);
       } else {
-        sap_push<0>(sb, nb, h, f);
-        sap_push<1>(sb, nb, h, f);
-        sap_push<2>(sb, nb, h, f);
-        sap_push<3>(sb, nb, h, f);
+        SU3<float> U;
+        sb.link(0, U);
+        sap_push<0>(sb, nb, h, f, U);
+        sap_push<1>(sb, nb, h, f, U);
+        sap_push<2>(sb, nb, h, f, U);
+        sap_push<3>(sb, nb, h, f, U);
       }
       // the half-spinors are complete; their writers need not wait
       if (SHV < 32) __syncthreads();
@@ -734,7 +748,7 @@ __global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
 // Right-hand sides per CTA of a batch.  A CTA that takes several stages the block once for all of them,
 // but too few CTAs leave SMs idle: the number of waves times the work of a CTA is made smallest (staging
 // costs about 0.1 of a block solve).  20 fields at 24x16^3 (192 blocks of a colour, 304 CTAs resident):
-// 3.41 ms; one CTA for all fields of a block 6.86 ms with the kernel this one replaced.
+// 3.35 ms; one CTA for all fields of a block 6.86 ms with the kernel this one replaced.
 inline int sap_rhs_per_cta(int nblocks, int nrhs, int slots) {
   int best = nrhs;
   double best_t = 1e300;
