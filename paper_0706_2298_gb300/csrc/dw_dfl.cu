@@ -396,6 +396,78 @@ __global__ void __launch_bounds__(128 * RK_G, sizeof(T) == 4 ? 2 : 1) restrict_n
   }
 }
 
+// c_r[L][k] = (phi^L_k, psi_r) for batches with the BF16 basis: a CTA takes RT right-hand sides of one deflation block
+// (the groups of a batch are neighbouring CTAs), so a basis value is read and unpacked once per RT of them.  One unit
+// of the basis (four components) at a time: RT x 4 field components, 4 basis components and 2 RT Ns / RK_G sums
+// stay within the 128 registers of 512 threads.  Bound: issue and the latency of the loads (16 warps per SM).  12 fields
+// of 24x16^3, Ns = 20: 100 us.
+template <int NS, int RT>
+__global__ void __launch_bounds__(128 * RK_G, 1) restrict_batch_kernel(Geom g, const int* __restrict__ sub, int nsub,
+                                                                        const uint4* __restrict__ b16,
+                                                                        const float* __restrict__ psi0,
+                                                                        float* __restrict__ c0, int nrhs,
+                                                                        size_t fstride, size_t cstride) {
+  static_assert(NS % RK_G == 0, "the groups share the basis vectors evenly");
+  constexpr int KP = NS / RK_G;
+  using WH = WarpHalve<float, 2 * KP, 16>;
+  constexpr int MF = WH::final_m();
+  __shared__ float sh[RT][4 * RK_G][2 * KP];
+  const int ngr = (nrhs + RT - 1) / RT;
+  const int L = blockIdx.x / ngr, r0 = (blockIdx.x - L * ngr) * RT, nr = min(RT, nrhs - r0);
+  const size_t V = g.V;
+  const int nsite = nsub * g.svol;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int grp = threadIdx.x >> 7, tl = threadIdx.x & 127, k0 = grp * KP;
+  cplx<float> acc[RT][KP];
+#pragma unroll
+  for (int r = 0; r < RT; ++r)
+#pragma unroll
+    for (int k = 0; k < KP; ++k) acc[r][k] = {0.f, 0.f};
+  for (int t = tl; t < nsite; t += 128) {
+    const size_t i = (size_t)dfl_site(g, sub, nsub, L, t);
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      cplx<float> p[RT][4];
+#pragma unroll
+      for (int r = 0; r < RT; ++r) {     // the missing fields of the last group: its last one again, not stored
+        const float4* f = reinterpret_cast<const float4*>(psi0 + (size_t)(r0 + min(r, nr - 1)) * fstride);
+        unpack_unit(__ldg(f + (2 * u) * V + i), p[r]);
+        unpack_unit(__ldg(f + (2 * u + 1) * V + i), p[r] + 2);
+      }
+#pragma unroll
+      for (int k = 0; k < KP; ++k) {
+        cplx<float> f[4];
+        bf16_unpack4(__ldg(b16 + ((size_t)(k0 + k) * 3 + u) * V + i), f);
+#pragma unroll
+        for (int r = 0; r < RT; ++r) {
+          cplx<float> s = {0.f, 0.f};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) cmacc(s, f[j], p[r][j]);
+          acc[r][k] += s;
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < RT; ++r) {
+    float x[2 * KP];
+#pragma unroll
+    for (int k = 0; k < KP; ++k) { x[2 * k] = acc[r][k].re; x[2 * k + 1] = acc[r][k].im; }
+    int base = 0;
+    WH::run(x, lane, base);
+#pragma unroll
+    for (int m = 0; m < MF; ++m) sh[r][w][base + m] = x[m];
+  }
+  __syncthreads();
+  if (tl < 2 * KP)
+    for (int r = 0; r < nr; ++r) {
+      float y = sh[r][4 * grp][tl];
+#pragma unroll
+      for (int q = 1; q < 4; ++q) y += sh[r][4 * grp + q][tl];
+      c0[(size_t)(r0 + r) * cstride + (size_t)L * 2 * NS + 2 * k0 + tl] = y;
+    }
+}
+
 // psi = mode 0: Phi c ; 1: psi + Phi c ; 2: psi - Phi c
 // A thread per site; CTAs of BLOCK threads.  FP32: 256 threads (4 KB pieces of the basis' unit planes) and 24
 // warps per SM: 78 us at 40x24x16x24, Ns = 20 (5.0 TB/s), 34 us at 24x16^3, Ns = 32; 128 threads 87 and 49 us,
@@ -430,6 +502,47 @@ __global__ void __launch_bounds__(BLOCK, sizeof(T) != 4 ? 1 : BLOCK == 256 ? 3 :
   }
   store_site<T, 12>(psi, V, i, out);
   }
+}
+
+// psi_r = Phi c_r for batches with the BF16 basis: a thread holds one site of RT right-hand sides (24 RT
+// accumulators), so a basis value is read and unpacked once per RT of them; the groups of a batch are neighbouring CTAs.  Bound: issue
+// (12 warps per SM).  12 fields of 24x16^3, Ns = 20: 81 us; this and the restriction
+// together took 377 us with one field after the other in a CTA and the basis from L2.
+template <int RT>
+__global__ void __launch_bounds__(128, 3) prolong_batch_kernel(Geom g, const int* __restrict__ sap2dfl, int Ns,
+                                                               const uint4* __restrict__ b16,
+                                                               const float* __restrict__ c0, float* __restrict__ psi0,
+                                                               int nrhs, size_t fstride, size_t cstride) {
+  const int ngr = (nrhs + RT - 1) / RT;
+  const int blk = blockIdx.x / ngr, r0 = (blockIdx.x - blk * ngr) * RT, nr = min(RT, nrhs - r0);
+  const size_t V = g.V, i = (size_t)blk * 128 + threadIdx.x;
+  if (i >= V) return;
+  const int L = __ldg(sap2dfl + (int)(i >> g.lsvol));
+  const float2* cc = reinterpret_cast<const float2*>(c0 + (size_t)r0 * cstride) + (size_t)L * Ns;
+  const size_t cs2 = cstride / 2;
+  cplx<float> out[RT][12];
+#pragma unroll
+  for (int r = 0; r < RT; ++r)
+#pragma unroll
+    for (int j = 0; j < 12; ++j) out[r][j] = {0.f, 0.f};
+#pragma unroll 2
+  for (int k = 0; k < Ns; ++k) {
+    float2 ck[RT];
+#pragma unroll
+    for (int r = 0; r < RT; ++r) ck[r] = __ldg(cc + min(r, nr - 1) * cs2 + k);   // missing fields: not stored
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      cplx<float> f[4];
+      bf16_unpack4(__ldg(b16 + ((size_t)k * 3 + u) * V + i), f);
+#pragma unroll
+      for (int r = 0; r < RT; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cmac(out[r][4 * u + j], cplx<float>{ck[r].x, ck[r].y}, f[j]);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < RT; ++r)
+    if (r < nr) store_site<float, 12>(psi0 + (size_t)(r0 + r) * fstride, V, i, out[r]);
 }
 
 // ------------------------------------------------------------------ little operator assembly (A.1), FP64
@@ -2080,11 +2193,24 @@ extern "C" void dfl_destroy(dfl_ctx* d) {
   delete d;
 }
 
+// right-hand sides per CTA of the batched restriction and prolongation (two of a batch of two)
+constexpr int RB = 4;
 template <typename T, int NS>
 static bool launch_restrict_ns(dfl_ctx* d, const T* psi, T* c, int nrhs, cudaStream_t s) {
   if constexpr (NS == 0 || !std::is_same<T, float>::value) {
     return false;
   } else {
+    if (nrhs > 1 && d->basis16) {
+      const size_t fs = (size_t)d->c->V * 24, cs = (size_t)d->N * 2;
+      constexpr int R4 = NS <= 20 ? RB : 2;               // above, the sums of four fields do not fit the registers
+      if (nrhs == 2)
+        restrict_batch_kernel<NS, 2><<<d->Nb, 128 * RK_G, 0, s>>>(d->c->g, d->d_sub, d->nsub, d->basis16, psi, c, nrhs,
+                                                                  fs, cs);
+      else
+        restrict_batch_kernel<NS, R4><<<(unsigned)(d->Nb * ((nrhs + R4 - 1) / R4)), 128 * RK_G, 0, s>>>(
+            d->c->g, d->d_sub, d->nsub, d->basis16, psi, c, nrhs, fs, cs);
+      return true;
+    }
     restrict_ns_kernel<T, NS><<<d->Nb, 128 * RK_G, 0, s>>>(d->c->g, d->d_sub, d->nsub,
                                                            d->basis16 ? nullptr : d->basis64, d->basis16, psi, c, nrhs,
                                                            (size_t)d->c->V * 24, (size_t)d->N * 2);
@@ -2107,6 +2233,19 @@ template <typename T>
 static int prolong_t(dfl_ctx* d, const T* c, T* psi, int mode, cudaStream_t s, int nrhs = 1) {
   const size_t V = d->c->V;
   const double* b64 = d->basis16 ? nullptr : d->basis64;
+  if constexpr (std::is_same<T, float>::value) {
+    if (nrhs > 1 && mode == 0 && d->basis16) {
+      const unsigned nb = (unsigned)((V + 127) / 128);
+      if (nrhs == 2)
+        prolong_batch_kernel<2><<<nb, 128, 0, s>>>(d->c->g, d->d_sap2dfl, d->Ns, d->basis16, c, psi, nrhs, V * 24,
+                                                   (size_t)d->N * 2);
+      else
+        prolong_batch_kernel<RB><<<nb * ((nrhs + RB - 1) / RB), 128, 0, s>>>(d->c->g, d->d_sap2dfl, d->Ns, d->basis16, c,
+                                                                             psi, nrhs, V * 24, (size_t)d->N * 2);
+      dw_note_launch();
+      return DW_OK;
+    }
+  }
   if (sizeof(T) == 4 && V / 256 >= 2 * (size_t)d->c->sms)
     prolong_kernel<T, 256><<<(unsigned)((V + 255) / 256), 256, 0, s>>>(d->c->g, d->d_sap2dfl, d->Ns, b64, d->basis16, c,
                                                                        psi, mode, nrhs, V * 24, (size_t)d->N * 2);
