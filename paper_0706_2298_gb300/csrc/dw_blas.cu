@@ -481,36 +481,55 @@ DW_D dd split_double(double x) {
   return {hi, sign ? -lo : lo};
 }
 
-__global__ void f64_to_dd_kernel(const double2* __restrict__ x, float4* __restrict__ y, size_t n2) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
-    const double2 v = x[i];
-    const dd a = split_double(v.x), b = split_double(v.y);
-    y[i] = make_float4(a.hi, a.lo, b.hi, b.lo);
-  }
-}
-__global__ void dd_to_f64_kernel(const float4* __restrict__ x, double2* y, size_t n2, int add) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 v = x[i];
-    double2 o = make_double2(widen(v.x) + widen(v.y), widen(v.z) + widen(v.w));
-    if (add) {
-      const double2 t = y[i];
-      o.x += t.x;
-      o.y += t.y;
+// Both conversions: four 16-byte loads in flight per thread.  Bound: DRAM and latency; with one load per thread at a
+// time the double-float D of 40x24x16x24, conversions included, took 375 us instead of 326.
+constexpr int CV = 4;
+__global__ void __launch_bounds__(256) f64_to_dd_kernel(const double2* __restrict__ x, float4* __restrict__ y, size_t n2) {
+  const size_t i0 = blockIdx.x * (size_t)(256 * CV) + threadIdx.x;
+  double2 v[CV];
+#pragma unroll
+  for (int k = 0; k < CV; ++k)
+    if (i0 + k * 256 < n2) v[k] = x[i0 + k * 256];
+#pragma unroll
+  for (int k = 0; k < CV; ++k)
+    if (i0 + k * 256 < n2) {
+      const dd a = split_double(v[k].x), b = split_double(v[k].y);
+      y[i0 + k * 256] = make_float4(a.hi, a.lo, b.hi, b.lo);
     }
-    y[i] = o;
-  }
 }
+__global__ void __launch_bounds__(256) dd_to_f64_kernel(const float4* __restrict__ x, double2* y, size_t n2, int add) {
+  const size_t i0 = blockIdx.x * (size_t)(256 * CV) + threadIdx.x;
+  float4 v[CV];
+  double2 t[CV];
+#pragma unroll
+  for (int k = 0; k < CV; ++k) {
+    const bool in = i0 + k * 256 < n2;
+    if (in) v[k] = x[i0 + k * 256];
+    t[k] = in && add ? y[i0 + k * 256] : make_double2(0.0, 0.0);
+  }
+#pragma unroll
+  for (int k = 0; k < CV; ++k)
+    if (i0 + k * 256 < n2) {
+      double2 o = make_double2(widen(v[k].x) + widen(v[k].y), widen(v[k].z) + widen(v[k].w));
+      if (add) {
+        o.x += t[k].x;
+        o.y += t[k].y;
+      }
+      y[i0 + k * 256] = o;
+    }
+}
+inline unsigned conv_grid(size_t n2) { return (unsigned)((n2 + 256 * CV - 1) / (256 * CV) + (n2 == 0)); }
 
 }  // namespace
 
 void f64_to_dd(const double* x, dd* y, size_t n_real, cudaStream_t s) {
   const size_t n2 = n_real / 2;
-  f64_to_dd_kernel<<<RGRID * 2, 256, 0, s>>>(reinterpret_cast<const double2*>(x), reinterpret_cast<float4*>(y), n2);
+  f64_to_dd_kernel<<<conv_grid(n2), 256, 0, s>>>(reinterpret_cast<const double2*>(x), reinterpret_cast<float4*>(y), n2);
   dw_note_launch();
 }
 void dd_to_f64(const dd* x, double* y, size_t n_real, int add, cudaStream_t s) {
   const size_t n2 = n_real / 2;
-  dd_to_f64_kernel<<<RGRID * 2, 256, 0, s>>>(reinterpret_cast<const float4*>(x), reinterpret_cast<double2*>(y), n2,
+  dd_to_f64_kernel<<<conv_grid(n2), 256, 0, s>>>(reinterpret_cast<const float4*>(x), reinterpret_cast<double2*>(y), n2,
                                             add);
   dw_note_launch();
 }
