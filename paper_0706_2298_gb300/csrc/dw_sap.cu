@@ -247,7 +247,7 @@ template <int SHV>
 struct SapCfg {
   static constexpr int NS = 2 * SHV;
   static constexpr bool TM = SHV >= 64;
-  [[maybe_unused]] static constexpr int TCOLS = SHV >= 128 ? 256 : 128;       // columns of a CTA: 128 per warp of a lane quarter
+  DW_HD static constexpr uint32_t tcols() { return SHV >= 128 ? 256 : 128; }   // columns of a CTA: 128 per warp of a lane quarter
   static constexpr int FIXED = TM ? NS * 144 : NS * 288;      // clover block 1, or the links
   static constexpr size_t bytes = (size_t)FIXED + (size_t)SHV * (12 + 6 + 12) * 16;
 };
@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
   if constexpr (Cfg::TM) {
     if (t < 32) {
       asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tm)),
-                   "r"((uint32_t)Cfg::TCOLS) : "memory");
+                   "r"(Cfg::tcols()) : "memory");
       asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -740,7 +740,7 @@ __global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
   }
   if constexpr (Cfg::TM) {
     if (t < 32)
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tm), "r"((uint32_t)Cfg::TCOLS)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tm), "r"(Cfg::tcols())
                    : "memory");
   }
 }
