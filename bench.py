@@ -62,9 +62,9 @@ PLAIN_COUNTS = os.path.join(ROOT, "paper_0706_2298_gb300", "plain_gcr_counts.jso
 
 # DRAM bytes per little-GCR iteration of the cooperative kernel, from one ncu capture of the
 # current kernel (dram__bytes_read.sum + dram__bytes_write.sum of one launch / its iterations):
-# 48x24^3, Ns = 20: (76.61 + 3.65) MB over 41 iterations (cold cache: the first iteration reads
+# 48x24^3, Ns = 20: (75.18 + 3.30) MB over 41 iterations (cold cache: the first iteration reads
 # the little operator from HBM, the rest hit L2).  Remove an entry when the kernel changes.
-LITTLE_TRAFFIC = {("24^3x48", 20): 80.84e6 / 41}
+LITTLE_TRAFFIC = {("24^3x48", 20): 78.48e6 / 41}
 
 
 def aggregate_ranks(t_ms, steps, world, device="cpu"):
@@ -510,7 +510,7 @@ def main():
     hbm, peak_kind = peaks()
     l2 = l2_copy_bandwidth(torch)
     fp32_peak = fp32_peak_tflops()
-    # dominant kernel: the cooperative little GCR (A.2-A.4).  Algorithmic bytes per little-GCR
+    # the cooperative little GCR (A.2-A.4), the largest kernel with a bandwidth bound.  Algorithmic bytes per little-GCR
     # iteration (FP32): the eight off-diagonal Ns x Ns blocks of every block row of the little
     # operator (both parities, read once by the two hops) and the 2 Ns global-mode vectors g, B^g
     # of the A.3 projection (Ne Ns complex each).  The operator (66 MB) is L2-resident.
@@ -519,13 +519,13 @@ def main():
     t_little = sum(i.t_little for i in infos)
     n_lit = sum(i.little_iterations for i in infos)
     lit_s = t_little / max(n_lit, 1)
-    roof = {"kernel": f"little_gcr_coop_kernel<float,{Ns}>", "bound": "l2", "achieved": lit_bytes / lit_s / 1e9,
+    roof = {"kernel": f"little_gcr_warp_kernel<{Ns}>", "bound": "l2", "achieved": lit_bytes / lit_s / 1e9,
             "peak": l2["gbs"], "unit": "GB/s", "frac": lit_bytes / lit_s / 1e9 / l2["gbs"],
             "traffic": LITTLE_TRAFFIC.get((args.workload, Ns)), "peak_kind": "measured here: " + l2["how"],
             "per": "little GCR iteration", "us_per_iteration": lit_s * 1e6, "algorithmic_bytes": lit_bytes,
             "l2_resident": True, "hbm_peak": hbm, "frac_of_hbm": lit_bytes / lit_s / 1e9 / hbm,
             "iterations_per_solve": n_lit / max(len(infos), 1)}
-    # the Schwarz block kernel (second largest): 960 algorithmic bytes per site processed
+    # the Schwarz block kernel (the largest share of the solve): 960 algorithmic bytes per site processed
     t_sap = sum(i.t_sap for i in infos)
     n_sap_launch = sum(i.iterations for i in infos) * 2 * wl["ncy"]
     sap_launch_s = t_sap / max(n_sap_launch, 1)

@@ -269,9 +269,9 @@ template void dirac_full<double>(dw_ctx*, const double*, double*, cudaStream_t);
 // clover blocks.  The double-float links are stored with all three rows: rebuilding the third one in
 // double-float arithmetic, in both halves, took a third of the operations, and the kernel uses a tenth of
 // the memory bandwidth.  The result leaves as FP64, D in or eta - D in.
-// Bound: FP32 issue and latency (20 warps per SM).  40x24x16x24, with the conversion of the input: 375 us;
-// unrolled over the directions 525 us, with the third row rebuilt and results and residual in passes of their
-// own 745 us; 4 CTAs per SM 3% more, 6 CTAs 10%.
+// Bound: FP32 issue and latency (20 warps per SM).  40x24x16x24, with the conversion of the input: 326 us;
+// with a conversion 49 us slower, unrolled over the directions 525 us, also with the third row rebuilt and results
+// and residual in passes of their own 745 us; 4 CTAs per SM 3% more, 6 CTAs 10%.
 constexpr int DD_BLOCKS = 5;      // CTAs per SM
 // s + e = a b for double-float a, b, exact up to the product of the low parts (Dekker's product of
 // the leading parts by one FMA); s + e += a b with the leading part added by TwoSum and all errors
