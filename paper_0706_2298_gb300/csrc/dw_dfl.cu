@@ -65,7 +65,6 @@ struct dfl_ctx {
   bool a3 = false;
   double* g64 = nullptr; float* g32 = nullptr;         // [Ns][Ne*Ns]
   double* Bg64 = nullptr; float* Bg32 = nullptr;       // B^ g
-  float* BgG32 = nullptr;                              // [Ns][Ns] = (B^ g_l, B^ g_m)
   std::vector<cd> Atil_inv;                            // Ns x Ns row-major
   std::vector<int> hlist0;                             // even blocks (host copy of d_list[0])
   std::vector<cd> graw;                                // [Ns][Ne*Ns] (phi^L_k, psi_l) on even blocks (A.3 input)
@@ -2199,7 +2198,7 @@ extern "C" void dfl_destroy(dfl_ctx* d) {
   if (!d) return;
   void* ptrs[] = {d->d_sub, d->d_sap2dfl, d->d_bnb, d->d_list[0], d->d_list[1], d->d_lnb[0], d->d_lnb[1],
                   d->basis64, d->basis16, d->B64, d->Binv64, d->Binv32, d->M64, d->M32, d->g64, d->g32,
-                  d->Bg64, d->Bg32, d->BgG32, d->lw[0], d->lw[1], d->B32, d->fw[0], d->fw[1], d->Ainv64, d->Ainv32,
+                  d->Bg64, d->Bg32, d->lw[0], d->lw[1], d->B32, d->fw[0], d->fw[1], d->Ainv64, d->Ainv32,
                   d->coop_partial, d->coop_out, d->ref64, d->ref32, d->ddf, d->ddl, d->mw, d->mio,
                   d->meo, d->macc, d->mscr, d->mtol, d->mout};
   for (void* p : ptrs)
@@ -2693,8 +2692,7 @@ static int little_gcr_coop(dfl_ctx* d, const T* b, T* v, double tol, int maxit, 
   size_t dsm = coop_dyn_smem<T>(d->coop_grid);
   if (sizeof(T) == 4 && d->coop_warp) {
     const LittleArgs l = {a.Ne, a.No, nkv, maxit, a.a3, a.list_e, a.list_o, a.lnb_e, a.lnb_o, (const float*)a.M,
-                          (const float*)a.g, (const float*)a.Bg, (const float*)a.Ainv, d->BgG32, (const float*)b,
-                          (float*)v,
+                          (const float*)a.g, (const float*)a.Bg, (const float*)a.Ainv, (const float*)b, (float*)v,
                           (float*)a.work, a.acc, a.out, tol};
     le = little_warp_launch(l, d->Ns, d->coop_grid, s);
   } else {
@@ -3406,8 +3404,6 @@ static int little_setup(dw_ctx* c, dfl_ctx* d, const double* B64_given) {
         DW_CUDA(cudaMalloc(&d->Ainv32, (size_t)Ns * Ns * 2 * sizeof(float)));
         DW_CUDA(cudaMemcpy(d->Ainv64, X.data(), (size_t)Ns * Ns * sizeof(cd), cudaMemcpyHostToDevice));
         blas_convert<double, float>(d->Ainv64, d->Ainv32, 1.0, (size_t)Ns * Ns, s);
-        DW_CUDA(cudaMalloc(&d->BgG32, (size_t)Ns * Ns * 2 * sizeof(float)));
-        little_gram(d->Bg64, ne, Ns, d->BgG32, s);
       }
     }
   }

@@ -10,18 +10,16 @@
 // The CTA's slices of g, B^ g and chi'_j stay in shared memory (where they fit), so the inner products and
 // updates of a step touch no L2.
 // Bound: latency and instruction issue of short phases at 4 warps per scheduler (16 warps of 128 registers;
-// L2 would deliver the 75 MB of an iteration in 4 us).  Time per iteration: Nb = 2592, Ns = 20: 21.5 us, with
-// a shared-memory ring of bulk copies and 8 warps 34.8 us; Nb = 384: 15.1 (20.5) us; Nb = 32, Ns = 16: 13.7
-// (18.7) us.  Two blocks in registers per warp spill and take 25.2 us, 8 warps with two blocks 24.1 us; blocks
-// kept in tensor memory or staged in shared memory save L2 reads that are not the bound (28 us: the code for
+// L2 would deliver the 75 MB of an iteration in 4 us).  Time per iteration: Nb = 2592, Ns = 20: 23.7 us, with
+// a shared-memory ring of bulk copies and 8 warps 34.8 us; Nb = 384: 16.7 (20.5) us; Nb = 32, Ns = 16: 14.6
+// (18.7) us.  Two blocks in registers per warp spill and cost 3.7 us more, 8 warps with two blocks 2.6 us; blocks
+// kept in tensor memory or staged in shared memory save L2 reads that are not the bound (6.5 us more: the code for
 // several sources of blocks costs more issue slots).
-// A step has two grid barriers: between its hops, and one reduction of all inner products with
-// c = B^ rho_k: (g_l, c), (B^ g_l, c), (chi'_j, c), (c, rho_k), |c|^2 and the CTA shares of |rho_k|^2.  With
-// the constant (B^ g_l, B^ g_m) and the tables (B^ g_l, chi'_j), (B^ g_l, rho_k) carried along, they give the
-// projection, the Gram-Schmidt coefficients, |chi'_k|^2 and (chi'_k, rho_k), so chi'_k and rho_{k+1} are
-// formed in one pass without a second reduction; when |chi'_k|^2 is so much smaller than |c|^2 that the
-// difference would lose digits, the two numbers are summed directly.  The residual of a step is not
-// published: the next hop forms rho_k = rho_{k-1} - alpha chi'_{k-1} from two published vectors.
+// A step has three grid barriers: between its hops, after c = B^ rho_k, where (g_l, c), (chi'_j, c) and the CTA
+// shares of |rho_k|^2 are reduced, and after chi'_k is formed, where (chi'_k, rho_k), |chi'_k|^2 and (B^ g_l, chi'_k)
+// are summed from chi'_k itself.  The coefficients of P~_L c on chi'_j follow from (chi'_j, c) and the stored
+// (B^ g_l, chi'_j).  The last barrier also publishes chi'_k, so that the residual of a step needs none of its own:
+// the next odd hop forms rho_{k+1} = rho_k - alpha chi'_k from the two vectors as it gathers them.
 // Reductions: FP64 atomics into one of three rotating accumulator sets, one grid barrier, then every CTA
 // reads the totals.  A value has four accumulators (a quarter of the CTAs each): the atomics on one address
 // are served one after the other, and 132 values of 152 CTAs take 3.5 us with one accumulator, 2.1 us with
@@ -57,11 +55,9 @@ struct LShared {
   cf beta[LITTLE_NKV];       // solution coefficients
   cf be[LITTLE_NKV][LITTLE_NKV];   // [j][k]: (chi'_j, P~_L c_k) / |chi'_j|^2
   cf tg[LITTLE_NKV][32];     // (B^ g_l, chi'_j) of the current cycle
-  cf q[32];                  // (B^ g_l, rho_k)
-  cf z[32], w[32];           // A~^{-1} g^+ c; (B^ g_l, P~_L c)
-  cf ainv[32 * 32], gram[32 * 32];   // A~^{-1}; (B^ g_l, B^ g_m), row-major
+  cf z[32];                  // A~^{-1} g^+ c
+  cf ainv[32 * 32];          // A~^{-1}, row-major
   cf ac;                     // alpha_{k-1}
-  float sc[4];               // |chi'_k|^2, (chi'_k, rho_k), whether they need a direct sum
   float rr;                  // this CTA's share of |rho_k|^2 (folded into the next reduction)
   int phase;
 };
@@ -305,7 +301,7 @@ size_t dyn_bytes(int rows, int nkv, bool vs) {
   if (vs) b += (size_t)(2 * NS + nkv) * rows * NS * sizeof(cf);
   return b;
 }
-constexpr size_t DYN_MAX = 194 * 1024;      // with the static part (31 KB) below 227 KB
+constexpr size_t DYN_MAX = 194 * 1024;      // with the static part (21 KB) below 227 KB
 
 template <int NS, bool VS>
 __global__ void __launch_bounds__(LT, 1) little_gcr_warp_kernel(LittleArgs a) {
@@ -323,7 +319,7 @@ __global__ void __launch_bounds__(LT, 1) little_gcr_warp_kernel(LittleArgs a) {
   const int CR = min(Rmax, LCH);
   cf* xs = reinterpret_cast<cf*>(dyn + ((size_t)18 * Rmax * sizeof(int) + 15) / 16 * 16);
   cf* hp = xs + CR * 8 * NS;
-  cf* ckS = hp + CR * 8 * NS;                            // c = B^ rho_k, rho_k, then (VS) g, B^ g, chi'_j: one array
+  cf* ckS = hp + CR * 8 * NS;                            // c = B^ rho_k, then chi'_k; rho_k; (VS) g, B^ g, chi'_j
   cf* rkS = ckS + Rmax * NS;
   const int len = even.n * NS;                           // entries of this CTA
   const size_t s0 = (size_t)even.first * NS;             // first of them in the global vectors
@@ -351,8 +347,8 @@ __global__ void __launch_bounds__(LT, 1) little_gcr_warp_kernel(LittleArgs a) {
   cg::grid_group grid = cg::this_grid();
   if (t == 0) sh.phase = 0;
   if (a.a3) {
-    const cf *Ai = reinterpret_cast<const cf*>(a.Ainv), *Gm = reinterpret_cast<const cf*>(a.BgG);
-    for (int e = t; e < NS * NS; e += LT) { sh.ainv[e] = Ai[e]; sh.gram[e] = Gm[e]; }
+    const cf* Ai = reinterpret_cast<const cf*>(a.Ainv);
+    for (int e = t; e < NS * NS; e += LT) sh.ainv[e] = Ai[e];
     if (VS)
       for (int e = t; e < NS * len; e += LT) {
         const int l = e / len, i = e - l * len;
@@ -363,7 +359,7 @@ __global__ void __launch_bounds__(LT, 1) little_gcr_warp_kernel(LittleArgs a) {
   __syncthreads();
   const float4* M = reinterpret_cast<const float4*>(a.M);
   Block<NS> buf;
-  const int na = a.a3 ? 2 * NS : 0;
+  const int nd = a.a3 ? NS : 0;                          // deflation vectors
   const cf zero = {0.f, 0.f};
   auto each = [&](auto&& f) {
     for (int i = t; i < len; i += LT) f(i);
@@ -395,7 +391,7 @@ __global__ void __launch_bounds__(LT, 1) little_gcr_warp_kernel(LittleArgs a) {
     project(ckS, bgV, -1.f);
     __syncthreads();
   };
-  // rho in ckS: published as rho_0 of a cycle; |rho|^2 and (B^ g_l, rho) reduced
+  // rho in ckS: published as rho_0 of a cycle; |rho|^2 reduced
   auto start_cycle = [&](cf* out, float* norm) {
     float s1[1] = {0.f};
     each([&](int i) {
@@ -406,11 +402,8 @@ __global__ void __launch_bounds__(LT, 1) little_gcr_warp_kernel(LittleArgs a) {
     });
     cta_sum<1>(sh, s1);
     if (t == 0) sh.rr = sh.cta[0];
-    if (a.a3) dots(sh, bgV, vn, NS, nullptr, 0, NS, ckS, len, 1);
-    reduce(grid, sh, 1 + na, a.acc);
-    if (a.a3 && t < NS) sh.q[t] = {sh.res[1 + 2 * t], sh.res[2 + 2 * t]};
+    reduce(grid, sh, 1, a.acc);
     *norm = sqrtf(sh.res[0]);
-    __syncthreads();
   };
 
   // rhsd = P~_L b, rho = rhsd, v = 0
@@ -433,79 +426,37 @@ __global__ void __launch_bounds__(LT, 1) little_gcr_warp_kernel(LittleArgs a) {
       cf* ck = chi(k) + s0;
       cf* xk = xi(k);
       each([&](int i) { xk[i] = rkS[i]; });              // xi_k = rho_k
+      // the odd hop reads rho_k of other CTAs as rho_{k-1} - alpha chi'_{k-1}: both were written before the last
+      // reduction's grid barrier
       const cf acs = k > 0 ? sh.ac : zero;
       hop<NS>(buf, M, odd, even, k > 0 ? rhob[cur ^ 1] : rhob[cur], k > 0 ? chi(k - 1) : nullptr, acs, xs, hp,
               [&](int e, cf s) { tmpo[(size_t)odd.first * NS + e] = s; });
       grid_barrier(grid);
       hop<NS>(buf, M, even, odd, tmpo, nullptr, zero, xs, hp, [&](int e, cf s) { ckS[e] = rkS[e] - s; });
-      // reduced: |c|^2, |rho_k|^2, (rho_k, c), then (g_l, c), (B^ g_l, c), (chi'_j, c)
-      if (VS && a.a3) {
-        dots(sh, ckS, vn, 2 + 2 * NS + k, nullptr, 0, 2 + 2 * NS + k, ckS, len, 0);
-      } else {
-        dots(sh, ckS, (size_t)Rmax * NS, 2, nullptr, 0, 2, ckS, len, 0);
-        if (a.a3) dots(sh, gV, vn, NS, bgV, vn, 2 * NS, ckS, len, 4);
-        dots(sh, chiV, vn, k, nullptr, 0, k, ckS, len, 4 + 2 * na);
-      }
-      __syncthreads();
-      if (t == 0) sh.cta[1] = sh.rr;
-      reduce(grid, sh, 4 + 2 * na + 2 * k, a.acc);
-      const float rn2 = sh.res[1], cc = sh.res[0];
+      // first reduction: |rho_k|^2, (g_l, c), (chi'_j, c)
+      dots(sh, gV, vn, nd, chiV, vn, nd + k, ckS, len, 1);
+      if (t == 0) sh.cta[0] = sh.rr;
+      reduce(grid, sh, 1 + 2 * (nd + k), a.acc);
+      const float rn2 = sh.res[0];
       rn = sqrtf(rn2);
       if (rn <= stop) break;                             // rho_k already converged: c unused
       // z = A~^{-1} (g, c)
-      const float* ru = sh.res + 4;
-      const float* rb = ru + na;
-      const float* re = ru + 2 * na;
-      if (a.a3) coarse<NS>(sh, ru);
+      const float* re = sh.res + 1 + 2 * nd;
+      if (a.a3) coarse<NS>(sh, sh.res + 1);
       __syncthreads();
-      // w_l = (B^ g_l, P~_L c) and beta_j = (chi'_j, P~_L c) / |chi'_j|^2
-      const int nw = a.a3 ? NS : 0;
-      small_rows(nw + k, [&](int r, int part) {
+      // beta_j = (chi'_j, P~_L c) / |chi'_j|^2, (chi'_j, P~_L c) = (chi'_j, c) - sum_l z_l (chi'_j, B^ g_l)
+      small_rows(k, [&](int j, int part) {
         cf s = zero;
-        if (a.a3 && r < nw + k) {
-          const cf* row = r < nw ? sh.gram + r * NS : sh.tg[r - nw];
-          for (int l = part; l < NS; l += LPART) {
-            const cf m = row[l];
-            cmac(s, sh.z[l], cf{m.re, r < nw ? m.im : -m.im});
-          }
-        }
+        if (j < k)
+          for (int l = part; l < nd; l += LPART) cmac(s, sh.z[l], conjg(sh.tg[j][l]));
         s = part_sum(s);
-        if (part == 0 && r < nw) sh.w[r] = {rb[2 * r] - s.re, rb[2 * r + 1] - s.im};
-        if (part == 0 && r >= nw && r < nw + k) {
-          const int j = r - nw;
+        if (part == 0 && j < k) {
           const float ic = 1.f / sh.c2[j];
           sh.be[j][k] = {(re[2 * j] - s.re) * ic, (re[2 * j + 1] - s.im) * ic};
         }
       });
       __syncthreads();
-      // |chi'_k|^2 = |c|^2 - Re sum conj(z_l) ((B^ g_l, c) + w_l) - sum |beta_j|^2 |chi'_j|^2,
-      // (chi'_k, rho_k) = (c, rho_k) - sum conj(z_l) (B^ g_l, rho_k)
-      if (t < 32) {
-        float n2 = 0.f, xr = 0.f, xm = 0.f;
-        if (t < nw) {
-          const cf z = sh.z[t], w = sh.w[t], q = sh.q[t];
-          n2 += z.re * (rb[2 * t] + w.re) + z.im * (rb[2 * t + 1] + w.im);
-          xr += z.re * q.re + z.im * q.im;
-          xm += z.re * q.im - z.im * q.re;
-        }
-        if (t < k) n2 += norm2(sh.be[t][k]) * sh.c2[t];
-        n2 = wsum(n2);
-        xr = wsum(xr);
-        xm = wsum(xm);
-        if (t == 0) {
-          sh.sc[0] = cc - n2;
-          sh.sc[1] = sh.res[2] - xr;                       // (c, rho_k) = conj (rho_k, c)
-          sh.sc[2] = -sh.res[3] - xm;
-          sh.sc[3] = cc - n2 < 1e-2f * cc ? 1.f : 0.f;
-        }
-      }
-      __syncthreads();
       // chi'_k = P~_L c - sum_j beta_j chi'_j
-      const bool direct = sh.sc[3] != 0.f;               // the same in all CTAs
-      cf alpha = zero;
-      if (!direct) alpha = {sh.sc[1] / sh.sc[0], sh.sc[2] / sh.sc[0]};
-      cf* rn1 = rhob[cur ^ 1] + s0;
-      float s1[1] = {0.f};
       float s3[3] = {0.f, 0.f, 0.f};
       for (int e0 = t & ~31; e0 < 2 * len; e0 += LT) {   // two threads per entry, whole warps
         const int e = e0 + (t & 31), i = min(e, 2 * len - 1) >> 1;
@@ -519,55 +470,35 @@ __global__ void __launch_bounds__(LT, 1) little_gcr_warp_kernel(LittleArgs a) {
         s.re += __shfl_xor_sync(0xffffffffu, s.re, 1);
         s.im += __shfl_xor_sync(0xffffffffu, s.im, 1);
         if (e < 2 * len && !(e & 1)) {
-          const cf y = ckS[i] - s;
-          cf r = rkS[i];
+          const cf y = ckS[i] - s, r = rkS[i];
           ck[i] = y;
           if (VS) chiV[(size_t)k * vn + i] = y;
-          if (direct) {
-            ckS[i] = y;
-            s3[0] += y.re * r.re + y.im * r.im;
-            s3[1] += y.re * r.im - y.im * r.re;
-            s3[2] += norm2(y);
-          } else {                                       // rho_{k+1} = rho_k - alpha chi'_k
-            cmsub(r, alpha, y);
-            rkS[i] = r;
-            rn1[i] = r;
-            s1[0] += norm2(r);
-          }
+          ckS[i] = y;
+          s3[0] += y.re * r.re + y.im * r.im;
+          s3[1] += y.re * r.im - y.im * r.re;
+          s3[2] += norm2(y);
         }
       }
-      float c2 = sh.sc[0];
-      cf ar = {sh.sc[1], sh.sc[2]};
-      if (direct) {                                      // the sums of chi'_k itself
-        cta_sum<3>(sh, s3);
-        reduce(grid, sh, 3, a.acc);
-        c2 = sh.res[2];
-        ar = {sh.res[0], sh.res[1]};
-        if (!(c2 > 0.f)) break;
-        alpha = {ar.re / c2, ar.im / c2};
-        each([&](int i) {
-          cf r = rkS[i];
-          cmsub(r, alpha, ckS[i]);
-          rkS[i] = r;
-          rn1[i] = r;
-          s1[0] += norm2(r);
-        });
-      }
-      // (B^ g_l, chi'_k) = w_l - sum_j beta_j (B^ g_l, chi'_j); (B^ g_l, rho_{k+1})
-      if (a.a3)
-        small_rows(NS, [&](int l, int part) {
-          cf s = zero;
-          if (l < NS)
-            for (int j = part; j < k; j += LPART) cmac(s, sh.be[j][k], sh.tg[j][l]);
-          s = part_sum(s);
-          if (part == 0 && l < NS) {
-            const cf x = sh.w[l] - s;
-            sh.tg[k][l] = x;
-            cf q = sh.q[l];
-            cmsub(q, alpha, x);
-            sh.q[l] = q;
-          }
-        });
+      // second reduction: (chi'_k, rho_k), |chi'_k|^2, (B^ g_l, chi'_k); its grid barrier publishes chi'_k, which the
+      // next odd hop gathers
+      cta_sum<3>(sh, s3);
+      dots(sh, bgV, vn, nd, nullptr, 0, nd, ckS, len, 3);
+      reduce(grid, sh, 3 + 2 * nd, a.acc);
+      const float c2 = sh.res[2];
+      const cf ar = {sh.res[0], sh.res[1]};
+      if (!(c2 > 0.f)) break;                            // the step is not used (zero or not a number)
+      // rho_{k+1} = rho_k - alpha chi'_k
+      const cf alpha = {ar.re / c2, ar.im / c2};
+      cf* rn1 = rhob[cur ^ 1] + s0;
+      float s1[1] = {0.f};
+      each([&](int i) {
+        cf r = rkS[i];
+        cmsub(r, alpha, ckS[i]);
+        rkS[i] = r;
+        rn1[i] = r;
+        s1[0] += norm2(r);
+      });
+      if (t < nd) sh.tg[k][t] = {sh.res[3 + 2 * t], sh.res[4 + 2 * t]};
       cta_sum<1>(sh, s1);
       if (t == 0) {
         sh.rr = sh.cta[0];
@@ -580,7 +511,7 @@ __global__ void __launch_bounds__(LT, 1) little_gcr_warp_kernel(LittleArgs a) {
       ++total;
       // |rho_{k+1}|^2 = |rho_k|^2 - |(chi'_k, rho_k)|^2 / |chi'_k|^2 (one step from the exact |rho_k|^2)
       const float est = rn2 - norm2(ar) / c2;
-      rn = est > 0 ? sqrtf(est) : 0.f;
+      rn = est <= 0.f ? 0.f : sqrtf(est);                // not a number stays one, and is not converged
       if (rn <= stop) { ++k; break; }
     }
     // v += sum_j y_j xi_j with y_j = alpha_j - sum_{i > j} beta_ji y_i: warp 0, lane i holds row i
@@ -627,26 +558,6 @@ __global__ void __launch_bounds__(LT, 1) little_gcr_warp_kernel(LittleArgs a) {
   }
 }
 
-__global__ void __launch_bounds__(128) gram_kernel(const double* __restrict__ X, size_t n, int Ns, float* G) {
-  const cplx<double>* a = reinterpret_cast<const cplx<double>*>(X) + (blockIdx.x / Ns) * n;
-  const cplx<double>* b = reinterpret_cast<const cplx<double>*>(X) + (blockIdx.x % Ns) * n;
-  cplx<double> s = {0.0, 0.0};
-  for (size_t i = threadIdx.x; i < n; i += 128) cmacc(s, a[i], b[i]);
-  __shared__ cplx<double> part[4];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    s.re += __shfl_xor_sync(0xffffffffu, s.re, o);
-    s.im += __shfl_xor_sync(0xffffffffu, s.im, o);
-  }
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    s = part[0] + part[1] + (part[2] + part[3]);
-    G[2 * blockIdx.x] = (float)s.re;
-    G[2 * blockIdx.x + 1] = (float)s.im;
-  }
-}
-
 template <int NS>
 bool ready(int grid, int sms) {
   int b = 0;
@@ -673,11 +584,6 @@ cudaError_t launch(const LittleArgs& a, int grid, cudaStream_t s) {
 }
 
 }  // namespace
-
-void little_gram(const double* X, size_t n, int Ns, float* G, cudaStream_t s) {
-  gram_kernel<<<Ns * Ns, 128, 0, s>>>(X, n, Ns, G);
-  dw_note_launch();
-}
 
 #define LITTLE_NS(NSRT, EXPR, OTHER)  \
   switch (NSRT) {                     \

@@ -6,7 +6,7 @@
 
 constexpr int LITTLE_NKV = 24;        // Krylov vectors per cycle, at most
 constexpr int LITTLE_COPIES = 4;      // accumulators of a value: CTA b adds to copy b mod 4
-constexpr int LITTLE_NV = 192;        // values per grid reduction, at most (4 Ns + 2 nkv + 4)
+constexpr int LITTLE_NV = 128;        // values per grid reduction, at most (2 Ns + 2 nkv + 3)
 
 constexpr size_t LITTLE_ACC_BYTES = (size_t)3 * LITTLE_COPIES * LITTLE_NV * sizeof(double);
 
@@ -14,7 +14,7 @@ struct LittleArgs {
   int Ne, No, nkv, maxit, a3;
   const int *list_e, *list_o, *lnb_e, *lnb_o;   // block rows of a parity; their neighbours' positions [row][8]
   const float *M;                               // [Nb][8][Ns][Ns] complex, column-major blocks
-  const float *g, *Bg, *Ainv, *BgG;             // [Ns][Ne Ns], [Ns][Ne Ns], [Ns][Ns], [Ns][Ns] = (B^ g_l, B^ g_m)
+  const float *g, *Bg, *Ainv;                   // [Ns][Ne Ns], [Ns][Ne Ns], [Ns][Ns]
   const float* b;
   float* v;
   float* work;                                  // 2 nkv + 5 vectors of Ne Ns complex
@@ -23,8 +23,6 @@ struct LittleArgs {
   double tol;
 };
 
-// G[l][m] = (X_l, X_m) of the Ns vectors X [Ns][n] complex, summed in FP64
-void little_gram(const double* X, size_t n, int Ns, float* G, cudaStream_t s);
 // whether a kernel for this Ns and number of block rows per CTA exists and `grid` CTAs of it are resident at
 // once (sets its attributes)
 bool little_warp_ready(int Ns, int rows, int grid, int sms);
