@@ -265,21 +265,43 @@ DW_D void tm_st2(uint32_t a, const float* v) {
                "r"(__float_as_uint(v[1])) : "memory");
 }
 DW_D void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// 18 consecutive columns; the registers are valid after tm_wait18, which every use of them depends on
-DW_D void tm_ld18(uint32_t a, float* v) {
+// Loads from tensor memory and the wait for them in one statement: their registers are undefined until the wait, and a
+// compiler may move or copy a value between two statements.
+// 2 x 18 consecutive columns
+DW_D void tm_ld36(uint32_t a, float* u, float* v) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%18];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%16,%17}, [%19];"
-      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
-        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]), "=f"(v[16]),
-        "=f"(v[17])
-      : "r"(a), "r"(a + 16));
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%36];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%16,%17}, [%37];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33}, [%38];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%34,%35}, [%39];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(u[0]), "=f"(u[1]), "=f"(u[2]), "=f"(u[3]), "=f"(u[4]), "=f"(u[5]), "=f"(u[6]), "=f"(u[7]), "=f"(u[8]),
+        "=f"(u[9]), "=f"(u[10]), "=f"(u[11]), "=f"(u[12]), "=f"(u[13]), "=f"(u[14]), "=f"(u[15]), "=f"(u[16]), "=f"(u[17]),
+        "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]), "=f"(v[16]), "=f"(v[17])
+      : "r"(a), "r"(a + 16), "r"(a + 18), "r"(a + 34));
 }
-DW_D void tm_wait18(float* v) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
-                 "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]),
-                 "+f"(v[16]), "+f"(v[17]));
+// 18 consecutive columns, and while they are on their way the spinor at shared address s (6 units, SHV apart)
+template <int SHV>
+DW_D void tm_ld18_spinor(uint32_t a, uint32_t s, float* v, float* p) {
+  constexpr int B = 16 * SHV;
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%42];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%16,%17}, [%43];\n\t"
+      "ld.shared.v4.f32 {%18,%19,%20,%21}, [%44];\n\t"
+      "ld.shared.v4.f32 {%22,%23,%24,%25}, [%44+%45];\n\t"
+      "ld.shared.v4.f32 {%26,%27,%28,%29}, [%44+%46];\n\t"
+      "ld.shared.v4.f32 {%30,%31,%32,%33}, [%44+%47];\n\t"
+      "ld.shared.v4.f32 {%34,%35,%36,%37}, [%44+%48];\n\t"
+      "ld.shared.v4.f32 {%38,%39,%40,%41}, [%44+%49];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]), "=f"(v[16]), "=f"(v[17]),
+        "=f"(p[0]), "=f"(p[1]), "=f"(p[2]), "=f"(p[3]), "=f"(p[4]), "=f"(p[5]), "=f"(p[6]), "=f"(p[7]), "=f"(p[8]),
+        "=f"(p[9]), "=f"(p[10]), "=f"(p[11]), "=f"(p[12]), "=f"(p[13]), "=f"(p[14]), "=f"(p[15]), "=f"(p[16]), "=f"(p[17]),
+        "=f"(p[18]), "=f"(p[19]), "=f"(p[20]), "=f"(p[21]), "=f"(p[22]), "=f"(p[23])
+      : "r"(a), "r"(a + 16), "r"(s), "n"(B), "n"(2 * B), "n"(3 * B), "n"(4 * B), "n"(5 * B)
+      : "memory");
 }
 
 // CTA barriers of a subset: wait for, or only announce, the arrival of n threads at barrier id
@@ -337,29 +359,37 @@ struct SapBlock {
       tm_wait_st();
     }
   }
-  // whole warps only (tensor memory); U may be used after link_wait
-  DW_D void link(int mu, SU3<float>& U) const {
-    cplx<float>* m = &U.m[0][0];
+  // the links of directions mu and mu + 1; whole warps only (tensor memory)
+  DW_D void link_pair(int mu, SU3<float>& U, SU3<float>& N) const {
     if constexpr (Cfg::TM) {
-      tm_ld18(tm + mu * 18, &m[0].re);
+      tm_ld36(tm + mu * 18, &U.m[0][0].re, &N.m[0][0].re);
     } else {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) unpack_unit(fix4[(mu * 4 + k) * NS + t], m + 2 * k);
-      const float2 l = fix2[mu * NS + t];
-      m[8] = {l.x, l.y};
+      link(mu, U);
+      link(mu + 1, N);
     }
   }
-  DW_D void link_wait(SU3<float>& U) const {
-    if constexpr (Cfg::TM) tm_wait18(&U.m[0][0].re);
+  // a link and the spinor of vec at site `at`; whole warps only (tensor memory)
+  DW_D void link_spinor(int mu, int at, SU3<float>& U, cplx<float>* f) const {
+    if constexpr (Cfg::TM) {
+      tm_ld18_spinor<SHV>(tm + mu * 18, smem_u32(vec + at), &U.m[0][0].re, &f[0].re);
+    } else {
+      link(mu, U);
+      get(vec, SHV, at, f);
+    }
+  }
+  // from shared memory
+  DW_D void link(int mu, SU3<float>& U) const {
+    cplx<float>* m = &U.m[0][0];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) unpack_unit(fix4[(mu * 4 + k) * NS + t], m + 2 * k);
+    const float2 l = fix2[mu * NS + t];
+    m[8] = {l.x, l.y};
   }
   // y = A_oo^{-1} x (odd) or A_ee x (even)
   DW_D void clover(size_t V, long long i, const cplx<float>* x, cplx<float>* y) const {
     cplx<float> s[18];
     if constexpr (Cfg::TM) {
-      tm_ld18(tm + 72, &s[0].re);
-      tm_ld18(tm + 90, &s[9].re);
-      tm_wait18(&s[0].re);
-      tm_wait18(&s[9].re);
+      tm_ld36(tm + 72, &s[0].re, &s[9].re);
       herm6_mul(s, x, y);
 #pragma unroll
       for (int k = 0; k < 9; ++k) unpack_unit(fix4[k * NS + t], s + 2 * k);
@@ -420,28 +450,21 @@ template <int MU, int SHV>
 DW_D void sap_forward(const SapBlock<SHV>& sb, const SapNb& nb, cplx<float>* acc) {
   SU3<float> U;
   cplx<float> p[12], w[6];
-  sb.link(MU, U);
-  sb.get(sb.vec, SHV, nb.at(2 * MU), p);       // some site of the block where the hop leaves it
-  sb.link_wait(U);
+  sb.link_spinor(MU, nb.at(2 * MU), U, p);     // some site of the block where the hop leaves it
   if (nb.in(2 * MU)) {
     half_spinor<MU, -1, false>(p, U, w);
     add_half<MU, -1>(w, acc);
   }
 }
-// half-spinors U_mu(y)^+ (1 + gamma_mu) psi(y) of the owner's spinor; U is the link of direction MU on its way,
-// and is left as that of MU + 1
+// half-spinor U_mu(y)^+ (1 + gamma_mu) psi(y) of the owner's spinor
 template <int MU, int SHV>
-DW_D void sap_push(const SapBlock<SHV>& sb, const SapNb& nb, int h, const cplx<float>* psi, SU3<float>& U) {
-  sb.link_wait(U);
-  SU3<float> next;
-  if (MU < 3) sb.link(MU + 1, next);
+DW_D void sap_push(const SapBlock<SHV>& sb, const SapNb& nb, int h, const cplx<float>* psi, const SU3<float>& U) {
   if (nb.in(2 * MU)) {
     cplx<float> w[6];
     half_spinor<MU, +1, true>(psi, U, w);
 #pragma unroll
     for (int k = 0; k < 3; ++k) sb.half[(MU * 3 + k) * SHV + h] = pack_unit(w + 2 * k);
   }
-  if (MU < 3) U = next;
 }
 // acc += the backward term of direction mu, from the half-spinor of x - mu
 template <int MU, int SHV>
@@ -629,12 +652,13 @@ __global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
         sap_forward<2>(sb, nb, a);
         sap_forward<3>(sb, nb, a);
       } else {
-        SU3<float> U;
-        sb.link(0, U);
+        SU3<float> U, N;
+        sb.link_pair(0, U, N);
         sap_push<0>(sb, nb, h, f, U);
-        sap_push<1>(sb, nb, h, f, U);
+        sap_push<1>(sb, nb, h, f, N);
+        sb.link_pair(2, U, N);
         sap_push<2>(sb, nb, h, f, U);
-        sap_push<3>(sb, nb, h, f, U);
+        sap_push<3>(sb, nb, h, f, N);
       }
       // the half-spinors are complete; their writers need not wait
       if (SHV < 32) __syncthreads();
@@ -739,6 +763,10 @@ __global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
     __syncthreads();             // the next right-hand side writes half, vec and xb
   }
   if constexpr (Cfg::TM) {
+    // every warp's tensor-memory accesses come before the columns are given back
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (t < 32)
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tm), "r"(Cfg::tcols())
                    : "memory");
