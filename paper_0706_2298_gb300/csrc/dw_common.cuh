@@ -317,39 +317,36 @@ DW_D void hop_acc(cplx<T>* acc, const cplx<T>* psi, const SU3<T>& U, T sign) {
 }
 
 // ---------------------------------------------------------------- clover
-// y = A x for one chiral block stored in 18 slots (see layout above).  LAST: the off-diagonal products are
-// summed first and the diagonal ones, the largest, added last, so that the sums round at the size of the
-// smaller terms (D in FP32: 6e-8 instead of 9e-8 from FP64, at the same speed).  The Schwarz kernels, at
-// their register limit, add to the diagonal products instead (the other order spills, 1.44 -> 2.40 ms).
-template <bool LAST = false, typename T>
-DW_D void herm6_mul(const cplx<T>* s, const cplx<T>* x, cplx<T>* y) {
-  const T d[6] = {s[0].re, s[0].im, s[1].re, s[1].im, s[2].re, s[2].im};
-  if (!LAST) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) y[i] = d[i] * x[i];
-  }
-  int k = 3;
+// y = A x for one chiral block stored in 18 slots (see layout above): the off-diagonal products are summed first
+// (herm6_off, on slots 3..17) and the diagonal ones, the largest, added last, so that the sums round at the size
+// of the smaller terms (D in FP32: 6e-8 instead of 9e-8 from FP64, at the same speed).
+template <typename T>
+DW_D void herm6_off(const cplx<T>* s, const cplx<T>* x, cplx<T>* y) {
+  int k = 0;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
 #pragma unroll
     for (int j = i + 1; j < 6; ++j) {
-      if (LAST && i == 0 && j == 1) y[0] = s[k] * x[j]; else cmac(y[i], s[k], x[j]);
-      if (LAST && i == 0) y[j] = cmulc(s[k], x[0]); else cmacc(y[j], s[k], x[i]);
+      if (i == 0 && j == 1) y[0] = s[k] * x[j]; else cmac(y[i], s[k], x[j]);
+      if (i == 0) y[j] = cmulc(s[k], x[0]); else cmacc(y[j], s[k], x[i]);
       ++k;
     }
   }
-  if (LAST) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) { rmac(y[i].re, d[i], x[i].re); rmac(y[i].im, d[i], x[i].im); }
-  }
 }
-template <bool LAST = false, typename T>
+template <typename T>
+DW_D void herm6_mul(const cplx<T>* s, const cplx<T>* x, cplx<T>* y) {
+  const T d[6] = {s[0].re, s[0].im, s[1].re, s[1].im, s[2].re, s[2].im};
+  herm6_off(s + 3, x, y);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) { rmac(y[i].re, d[i], x[i].re); rmac(y[i].im, d[i], x[i].im); }
+}
+template <typename T>
 DW_D void clover_apply(const T* __restrict__ clov, size_t V, size_t i, const cplx<T>* x, cplx<T>* y) {
   cplx<T> s[18];
   load_site<T, 18>(clov, V, i, s);
-  herm6_mul<LAST>(s, x, y);
+  herm6_mul(s, x, y);
   load_site<T, 18>(clov + 36 * V, V, i, s);
-  herm6_mul<LAST>(s, x + 6, y + 6);
+  herm6_mul(s, x + 6, y + 6);
 }
 
 // ---------------------------------------------------------------- contexts

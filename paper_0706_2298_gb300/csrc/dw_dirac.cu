@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) dirac_full_kernel
   SiteRef s = decode(g, i);
   cplx<T> psi[12], y[12], acc[12];
   load_site<T, 12>(in, V, i, psi);
-  clover_apply<true>(clov, V, i, psi, y);
+  clover_apply(clov, V, i, psi, y);
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = {T(0), T(0)};
   hop_all(g, s, i, links, in, acc);
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) dirac_interleaved
   SiteRef s = decode(g, i);
   cplx<T> psi[12], y[12], acc[12];
   load_site<T, 12>(in, V, i, psi);
-  clover_apply<true>(clov, V, i, psi, y);
+  clover_apply(clov, V, i, psi, y);
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = {T(0), T(0)};
   hop_all(g, s, i, links, in, acc);
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(128) schur_odd_kernel(Geom g, const T* __restr
   hop_all(g, s, i, links, in, acc);
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = T(-0.5) * acc[k];
-  clover_apply<true>(clovinv, V, i, acc, v);
+  clover_apply(clovinv, V, i, acc, v);
   store_site<T, 12>(t, V, i, v);
 }
 
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(128) schur_even_kernel(Geom g, const T* __rest
   long long i = site_index(g, s.b, 0, s.h);
   cplx<T> psi[12], y[12], acc[12];
   load_site<T, 12>(in, V, i, psi);
-  clover_apply<true>(clov, V, i, psi, y);
+  clover_apply(clov, V, i, psi, y);
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = {T(0), T(0)};
   hop_all(g, s, i, links, t, acc);
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(128) clover_inv_odd_kernel(Geom g, const T* __
   long long i = site_index(g, b, 1, h);
   cplx<T> x[12], y[12];
   load_site<T, 12>(in, V, i, x);
-  clover_apply<true>(clovinv, V, i, x, y);
+  clover_apply(clovinv, V, i, x, y);
   store_site<T, 12>(t, V, i, y);
 }
 
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(128) eo_reconstruct_kernel(Geom g, const T* __
   hop_all(g, s, io, links, x, acc);
 #pragma unroll
   for (int k = 0; k < 12; ++k) y[k] += T(0.5) * acc[k];
-  clover_apply<true>(clovinv, V, io, y, z);
+  clover_apply(clovinv, V, io, y, z);
   store_site<T, 12>(out, V, io, z);
   load_site<T, 12>(x, V, ie, y);
   store_site<T, 12>(out, V, ie, y);
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(128) dirac_mrhs_kernel(Geom g, const T* __rest
       if (r < nr) {
         cplx<T> psi[12], y[12];
         load_site<T, 12>(in + (size_t)(r0 + r) * fstride, V, i, psi);
-        clover_apply<true>(clov, V, i, psi, y);
+        clover_apply(clov, V, i, psi, y);
 #pragma unroll
         for (int k = 0; k < 12; ++k) y[k] -= T(0.5) * acc[r][k];
         store_site<T, 12>(out + (size_t)(r0 + r) * fstride, V, i, y);

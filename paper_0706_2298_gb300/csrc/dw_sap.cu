@@ -238,10 +238,12 @@ __global__ void __launch_bounds__(SHV) sap_block_kernel(Geom g, const T* __restr
 // (tcgen05.st / tcgen05.ld 32x32b: a thread's columns of its lane), the other chiral block, the vector,
 // the half-spinors and x_e / b_o in shared memory: a block solve reads nothing from L2 between its first
 // and last access.  Smaller blocks keep the links in shared memory and read the clover term from L2.
-// While the odd sites apply A_oo^{-1}, the even ones apply A_ee.
+// While the odd sites apply A_oo^{-1}, the even ones apply A_ee.  The diagonal of the clover term, the largest part
+// of the block operator, is added to each sum last: 1.1e-7 from FP64 (4 cycles of 4 steps), 1.5e-7 with the hops added to
+// A_ee r^, at the same speed.
 // Bound: instruction issue and latency (16 warps per SM at 128 registers and 98 KB, issue slots 57% busy);
 // the rest is the two parities waiting for each other and tensor-memory loads.  48x24^3 on 4^4 blocks, 4
-// cycles of 4 steps: 1.42 ms (22 TFLOP/s); links in shared memory and the whole clover term in tensor
+// cycles of 4 steps: 1.40 ms (22 TFLOP/s); links in shared memory and the whole clover term in tensor
 // memory 1.60 ms; pulling both hop terms from shared memory with one thread per (site pair, spin) 1.78 ms.
 template <int SHV>
 struct SapCfg {
@@ -280,6 +282,27 @@ DW_D void tm_ld36(uint32_t a, float* u, float* v) {
         "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
         "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]), "=f"(v[16]), "=f"(v[17])
       : "r"(a), "r"(a + 16), "r"(a + 18), "r"(a + 34));
+}
+// 30 and 6 consecutive columns
+DW_D void tm_ld30(uint32_t a, float* v) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%30];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%31];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%24,%25,%26,%27}, [%32];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%28,%29}, [%33];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]), "=f"(v[9]),
+        "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]), "=f"(v[16]), "=f"(v[17]), "=f"(v[18]), "=f"(v[19]),
+        "=f"(v[20]), "=f"(v[21]), "=f"(v[22]), "=f"(v[23]), "=f"(v[24]), "=f"(v[25]), "=f"(v[26]), "=f"(v[27]), "=f"(v[28]), "=f"(v[29])
+      : "r"(a), "r"(a + 16), "r"(a + 24), "r"(a + 28));
+}
+DW_D void tm_ld6(uint32_t a, float* v) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%6];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%4,%5}, [%7];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5])
+      : "r"(a), "r"(a + 4));
 }
 // 18 consecutive columns, and while they are on their way the spinor at shared address s (6 units, SHV apart)
 template <int SHV>
@@ -385,18 +408,41 @@ struct SapBlock {
     const float2 l = fix2[mu * NS + t];
     m[8] = {l.x, l.y};
   }
-  // y = A_oo^{-1} x (odd) or A_ee x (even)
-  DW_D void clover(size_t V, long long i, const cplx<float>* x, cplx<float>* y) const {
-    cplx<float> s[18];
+  // The clover term, A_oo^{-1} (odd) or A_ee (even), in two parts, so that the diagonal products, the largest, can be
+  // added last: y = its off-diagonal part times x, and its diagonal d[12]
+  DW_D void clover_off(size_t V, long long i, const cplx<float>* x, cplx<float>* y) const {
+    cplx<float> s[16];                                    // s[0]: the last diagonal pair, unused
     if constexpr (Cfg::TM) {
-      tm_ld36(tm + 72, &s[0].re, &s[9].re);
-      herm6_mul(s, x, y);
+      tm_ld30(tm + 78, &s[1].re);
+      herm6_off(s + 1, x, y);
 #pragma unroll
-      for (int k = 0; k < 9; ++k) unpack_unit(fix4[k * NS + t], s + 2 * k);
-      herm6_mul(s, x + 6, y + 6);
+      for (int k = 0; k < 8; ++k) unpack_unit(fix4[(k + 1) * NS + t], s + 2 * k);
+      herm6_off(s + 1, x + 6, y + 6);
     } else {
-      clover_apply(cl, V, i, x, y);
+      const float4* q = reinterpret_cast<const float4*>(cl) + i;
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) unpack_unit(__ldg(q + (size_t)(9 * b + k + 1) * V), s + 2 * k);
+        herm6_off(s + 1, x + 6 * b, y + 6 * b);
+      }
     }
+  }
+  DW_D void clover_diag(size_t V, long long i, float* d) const {
+    float4 u[2];
+    if constexpr (Cfg::TM) {
+      tm_ld6(tm + 72, d);
+      u[0] = fix4[t];
+      u[1] = fix4[NS + t];
+    } else {
+      const float4* q = reinterpret_cast<const float4*>(cl) + i;
+      u[0] = __ldg(q);
+      u[1] = __ldg(q + V);
+      d[0] = u[0].x; d[1] = u[0].y; d[2] = u[0].z; d[3] = u[0].w; d[4] = u[1].x; d[5] = u[1].y;
+      u[0] = __ldg(q + 9 * V);
+      u[1] = __ldg(q + 10 * V);
+    }
+    d[6] = u[0].x; d[7] = u[0].y; d[8] = u[0].z; d[9] = u[0].w; d[10] = u[1].x; d[11] = u[1].y;
   }
   DW_D void put(float4* a, int stride, int at, const cplx<float>* f) const {
 #pragma unroll
@@ -634,9 +680,14 @@ __global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
     for (int k = 0; k < 12; ++k) a[k] = {0.f, 0.f};
     if (p) {                                  // b_o aside, t_o = A_oo^{-1} b_o
       sb.put(sb.xb, NS, t, f);
-      sb.clover(V, i, f, a);
+      float d[12];
+      sb.clover_off(V, i, f, a);
+      sb.clover_diag(V, i, d);
 #pragma unroll
-      for (int k = 0; k < 12; ++k) { f[k] = a[k]; a[k] = {0.f, 0.f}; }
+      for (int k = 0; k < 12; ++k) {
+        f[k] = {fmaf(d[k], f[k].re, a[k].re), fmaf(d[k], f[k].im, a[k].im)};
+        a[k] = {0.f, 0.f};
+      }
       sb.put(sb.vec, SHV, h, f);
     } else {
       sb.put(sb.xb, NS, t, a);                // x_e = 0
@@ -672,7 +723,7 @@ __global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
       }
       if (dst) {
         // odd: t_o = -1/2 A_oo^{-1} hops, or at the end x_o = A_oo^{-1}(b_o + 1/2 hops);
-        // even: 2 A_ee r^ (doubled: the hops added to it are halved below)
+        // even: the off-diagonal part of 2 A_ee r^ (doubled: the hops added to it are halved below)
         cplx<float> y[12];
         if (p) {
           if (s == last) sb.get(sb.xb, NS, t, f);
@@ -680,11 +731,18 @@ __global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
           for (int k = 0; k < 12; ++k) f[k] = s == last ? f[k] + 0.5f * a[k] : -0.5f * a[k];
         }
         if (p || s < last) {
-          sb.clover(V, i, f, y);
+          sb.clover_off(V, i, f, y);
+          if (p) {
+            float d[12];
+            sb.clover_diag(V, i, d);
 #pragma unroll
-          for (int k = 0; k < 12; ++k) {
-            if (p) { f[k] = y[k]; a[k] = {0.f, 0.f}; }
-            else a[k] = 2.f * y[k];
+            for (int k = 0; k < 12; ++k) {
+              f[k] = {fmaf(d[k], f[k].re, y[k].re), fmaf(d[k], f[k].im, y[k].im)};
+              a[k] = {0.f, 0.f};
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) a[k] = 2.f * y[k];
           }
         }
         if (s == last) break;
@@ -698,9 +756,11 @@ __global__ void __launch_bounds__(2 * SHV, 256 / SHV) sap_staged_kernel(
         } else {                              // minimal-residual step with p = A_ee r^ - D_eo t_o = a / 2
           float pr = 0.f, pi = 0.f, pp = 0.f;
           if (!p) {
+            float d[12];
+            sb.clover_diag(V, i, d);
 #pragma unroll
-            for (int k = 0; k < 12; ++k) {
-              a[k] = 0.5f * a[k];
+            for (int k = 0; k < 12; ++k) {                // the largest term of p, d r^, is added last
+              a[k] = {fmaf(d[k], f[k].re, 0.5f * a[k].re), fmaf(d[k], f[k].im, 0.5f * a[k].im)};
               pr += a[k].re * f[k].re + a[k].im * f[k].im;
               pi += a[k].re * f[k].im - a[k].im * f[k].re;
               pp += a[k].re * a[k].re + a[k].im * a[k].im;
