@@ -369,11 +369,12 @@ __global__ void __launch_bounds__(128 * RK_G, sizeof(T) == 4 ? 2 : 1) restrict_n
       load_site<T, 12>(psi, V, i, p);
 #pragma unroll
       for (int k = 0; k < KP; ++k) {
-        cplx<T> f[12], s = {T(0), T(0)};
+        // two chains: a sum of 24 products in one rounds at the size of the whole sum up to 24 times
+        cplx<T> f[12], s0 = {T(0), T(0)}, s1 = s0;
         load_basis<T>(b64, b16, V, k0 + k, i, f);
 #pragma unroll
-        for (int j = 0; j < 12; ++j) cmacc(s, f[j], p[j]);
-        acc[k] += s;
+        for (int j = 0; j < 6; ++j) { cmacc(s0, f[j], p[j]); cmacc(s1, f[j + 6], p[j + 6]); }
+        acc[k] += s0 + s1;
       }
     }
     T x[2 * KP];
@@ -439,9 +440,9 @@ __global__ void __launch_bounds__(128 * RK_G, 1) restrict_batch_kernel(Geom g, c
         bf16_unpack4(__ldg(b16 + ((size_t)(k0 + k) * 3 + u) * V + i), f);
 #pragma unroll
         for (int r = 0; r < RT; ++r) {
-          cplx<float> s = {0.f, 0.f};
+          cplx<float> s = cmulc(f[0], p[r][0]);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) cmacc(s, f[j], p[r][j]);
+          for (int j = 1; j < 4; ++j) cmacc(s, f[j], p[r][j]);
           acc[r][k] += s;
         }
       }
@@ -497,7 +498,7 @@ __global__ void __launch_bounds__(BLOCK, sizeof(T) != 4 ? 1 : BLOCK == 256 ? 3 :
     if (mode == 2) ck = -ck;
     load_basis<T>(b64, b16, V, k, i, f);
 #pragma unroll
-    for (int j = 0; j < 12; ++j) cmac(out[j], ck, f[j]);
+    for (int j = 0; j < 12; ++j) out[j] += ck * f[j];      // one rounding per term at the size of the sum
   }
   store_site<T, 12>(psi, V, i, out);
   }
@@ -524,21 +525,37 @@ __global__ void __launch_bounds__(128, 3) prolong_batch_kernel(Geom g, const int
   for (int r = 0; r < RT; ++r)
 #pragma unroll
     for (int j = 0; j < 12; ++j) out[r][j] = {0.f, 0.f};
-#pragma unroll 2
-  for (int k = 0; k < Ns; ++k) {
-    float2 ck[RT];
+  // two basis vectors at a time, their terms summed before they are added to the result: fewer roundings at its size than
+  // one chain, for fewer instructions than a sum per term; the last one of an odd Ns by itself
+  auto add = [&](int k, auto nk) {
+    constexpr int NK = decltype(nk)::value;
+    cplx<float> ck[NK][RT];
 #pragma unroll
-    for (int r = 0; r < RT; ++r) ck[r] = __ldg(cc + min(r, nr - 1) * cs2 + k);   // missing fields: not stored
+    for (int q = 0; q < NK; ++q)
+#pragma unroll
+      for (int r = 0; r < RT; ++r) {                       // missing fields: not stored
+        const float2 x = __ldg(cc + min(r, nr - 1) * cs2 + k + q);
+        ck[q][r] = {x.x, x.y};
+      }
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
-      cplx<float> f[4];
-      bf16_unpack4(__ldg(b16 + ((size_t)k * 3 + u) * V + i), f);
+      cplx<float> f[NK][4];
+#pragma unroll
+      for (int q = 0; q < NK; ++q) bf16_unpack4(__ldg(b16 + ((size_t)(k + q) * 3 + u) * V + i), f[q]);
 #pragma unroll
       for (int r = 0; r < RT; ++r)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cmac(out[r][4 * u + j], cplx<float>{ck[r].x, ck[r].y}, f[j]);
+        for (int j = 0; j < 4; ++j) {
+          cplx<float> s = ck[0][r] * f[0][j];
+          if (NK > 1) cmac(s, ck[NK - 1][r], f[NK - 1][j]);
+          out[r][4 * u + j] += s;
+        }
     }
-  }
+  };
+  int k = 0;
+#pragma unroll 1
+  for (; k + 1 < Ns; k += 2) add(k, std::integral_constant<int, 2>());
+  if (k < Ns) add(k, std::integral_constant<int, 1>());
 #pragma unroll
   for (int r = 0; r < RT; ++r)
     if (r < nr) store_site<float, 12>(psi0 + (size_t)(r0 + r) * fstride, V, i, out[r]);
