@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "../../include/dwsolve.h"
+#include "dw_host.cuh"
 
 #define DW_HD __host__ __device__ __forceinline__
 #define DW_D __device__ __forceinline__
@@ -422,6 +423,17 @@ struct dw_ctx {
 // synchronisation returns the memory to the driver and the next call maps it again (0.5 ms).  The pool goes
 // with dw_release_workspace and dw_destroy.
 cudaError_t dw_pool_alloc(dw_ctx* c, size_t bytes, void** p, cudaStream_t s);
+
+// the dynamic shared memory limit of a kernel on the current device, set at its first launch there
+template <auto KERNEL>
+cudaError_t dw_smem_limit(size_t bytes) {
+  static DeviceOnce once;
+  int device = 0;
+  if (const cudaError_t e = cudaGetDevice(&device)) return e;
+  return once(device, [&] {
+    return cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
+}
 
 // DW_OK when the calling thread's current device is the context's device; otherwise DW_EINVAL
 // with a message naming the entry point (kernels would mix memory of two devices).

@@ -364,16 +364,10 @@ __global__ void ptnet_adam_kernel(size_t n, float* w, const float* gr, float* m,
   w[t] -= lr * (mt / c1) / (sqrtf(vt / c2) + eps);
 }
 
-// dynamic shared memory of a kernel above the 48 KB default, once per kernel
-template <typename F>
-cudaError_t pt_attr(F* f, size_t bytes) {
-  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
 // nf fields: NI channels each in, 16 out (ADJ: the adjoint of a 16 -> NI layer)
 template <int NI, bool ADJ>
 cudaError_t launch_layer(dw_ctx* c, const float2* W, const float* in, float* out, int nf, cudaStream_t st) {
-  static const cudaError_t attr = pt_attr(ptnet_layer_kernel<NI, ADJ>, PtLayer<NI>::bytes);
-  if (attr != cudaSuccess) return attr;
+  if (const cudaError_t e = dw_smem_limit<ptnet_layer_kernel<NI, ADJ>>(PtLayer<NI>::bytes)) return e;
   const unsigned tiles = (unsigned)(c->V / PT_S * nf);
   ptnet_layer_kernel<NI, ADJ><<<tiles, PT_THREADS, PtLayer<NI>::bytes, st>>>(c->g, (const float*)c->links[DW_F32], W,
                                                                              in, out);
@@ -383,8 +377,7 @@ cudaError_t launch_layer(dw_ctx* c, const float2* W, const float* in, float* out
 // 16 channels in, 1 out; z: 9 scratch fields per field
 cudaError_t launch_layer_last(dw_ctx* c, const float2* W, const float* in, float* z, float* out, int nf,
                               cudaStream_t st) {
-  static const cudaError_t attr = pt_attr(ptnet_contract_kernel, PT_Z_BYTES);
-  if (attr != cudaSuccess) return attr;
+  if (const cudaError_t e = dw_smem_limit<ptnet_contract_kernel>(PT_Z_BYTES)) return e;
   ptnet_contract_kernel<<<(unsigned)(c->V / PT_S * nf), 32 * PT_ZW, PT_Z_BYTES, st>>>(c->g, W, in, z);
   dw_note_launch();
   ptnet_collect_kernel<<<(unsigned)(c->V / 128 * nf), 128, 0, st>>>(c->g, (const float*)c->links[DW_F32], z, out);
@@ -398,8 +391,7 @@ int pt_chunks(const dw_ctx* c, long long tiles, int ndir) {
 template <int MODE>
 cudaError_t launch_dw(dw_ctx* c, const float* local, const float* moved, float2* partial, float2* grad, int nf,
                       cudaStream_t st) {
-  static const cudaError_t attr = pt_attr(ptnet_dw_kernel<MODE>, PtDw<MODE>::bytes);
-  if (attr != cudaSuccess) return attr;
+  if (const cudaError_t e = dw_smem_limit<ptnet_dw_kernel<MODE>>(PtDw<MODE>::bytes)) return e;
   constexpr int E = MODE == 0 ? 4096 : 256, ND = MODE == 0 ? 9 : 1;
   const long long tiles = c->V / PT_S * nf;
   const int nc = pt_chunks(c, tiles, ND);
@@ -639,11 +631,7 @@ __global__ void __launch_bounds__(TC_THREADS, TcTile<S>::MIN_BLOCKS) ptnet_tc_la
 template <bool ADJ, int S>
 static int launch_tc(dw_ctx* c, const __nv_bfloat16* A, const float* in, float* out, int* err, cudaStream_t st) {
   using TT = TcTile<S>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    DW_CUDA(cudaFuncSetAttribute(ptnet_tc_layer_kernel<ADJ, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TT::SMEM));
-    attr_set = true;
-  }
+  DW_CUDA((dw_smem_limit<ptnet_tc_layer_kernel<ADJ, S>>(TT::SMEM)));
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

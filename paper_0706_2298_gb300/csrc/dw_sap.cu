@@ -853,13 +853,10 @@ template <int SHV>
 bool launch_sap_staged(dw_ctx* c, int colour, const float* rsrc, float* rdst, const float* dprev, float* dout,
                        float* xi, int first, int nmr, cudaStream_t st, int nrhs = 1) {
   constexpr size_t smem = SapCfg<SHV>::bytes;
-  static int state = 0;   // 0 unknown, 1 ok, -1 unavailable
-  if (state == 0) {
-    cudaError_t e = cudaFuncSetAttribute(sap_staged_kernel<SHV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    state = e == cudaSuccess ? 1 : -1;
+  if (dw_smem_limit<sap_staged_kernel<SHV>>(smem) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
   }
-  if (state < 0) return false;
   const int* list = c->d_colour_list + (colour ? c->ncolour[0] : 0);
   const int slots = c->sms * (256 / SHV);                                // resident CTAs (launch bounds)
   const int rpc = sap_rhs_per_cta(c->ncolour[colour], nrhs, slots);
@@ -878,11 +875,7 @@ void launch_sap(dw_ctx* c, int colour, const T* rsrc, T* rdst, const T* dprev, T
   constexpr int P = prec_of<T>();
   const int* list = c->d_colour_list + (colour ? c->ncolour[0] : 0);
   constexpr size_t smem = 3 * 12 * SHV * sizeof(cplx<T>);
-  static bool attr_set = false;   // per instantiation
-  if (!attr_set) {
-    cudaFuncSetAttribute(sap_block_kernel<T, SHV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr_set = true;
-  }
+  dw_smem_limit<sap_block_kernel<T, SHV>>(smem);         // a failure shows at the launch
   sap_block_kernel<T, SHV><<<c->ncolour[colour], SHV, smem, st>>>(c->g, (const T*)c->links[P], (const T*)c->clov[P],
                                                               (const T*)c->clovinv[P], list, rsrc, rdst, dprev,
                                                               dout, xi, first, nmr); dw_note_launch();
