@@ -340,7 +340,7 @@ struct WarpHalve {
 // threads, each for a quarter of the basis vectors and all sites of the block; per-thread partial sums, CTA
 // sum by warp halving + shared memory.
 // Bound: HBM (the basis).  A thread with all Ns vectors needs 2 Ns accumulators and 32 KB of unrolled code, and
-// 16 warps per SM did not keep enough loads in flight: 40x24x16x24, Ns = 20: 97 -> 79 us (4.9 TB/s); two groups 91 us.
+// 16 warps per SM did not keep enough loads in flight: 40x24x16x24, Ns = 20: 97 -> 81 us (4.8 TB/s); two groups 91 us.
 constexpr int RK_G = 4;
 template <typename T, int NS>
 __global__ void __launch_bounds__(128 * RK_G, sizeof(T) == 4 ? 2 : 1) restrict_ns_kernel(Geom g, const int* __restrict__ sub, int nsub,
@@ -470,10 +470,10 @@ __global__ void __launch_bounds__(128 * RK_G, 1) restrict_batch_kernel(Geom g, c
 
 // psi = mode 0: Phi c ; 1: psi + Phi c ; 2: psi - Phi c
 // A thread per site; CTAs of BLOCK threads.  FP32: 256 threads (4 KB pieces of the basis' unit planes) and 24
-// warps per SM: 78 us at 40x24x16x24, Ns = 20 (5.0 TB/s), 34 us at 24x16^3, Ns = 32; 128 threads 87 and 49 us,
-// but they fill the chip on lattices below 2 x 256 sites per SM (16^4, Ns = 12: 8.7 against 10.6 us).
+// warps per SM: 66 us at 40x24x16x24, Ns = 20 (5.9 TB/s), 17 us at 24x16^3; 128 threads 69 and 23 us, but their smaller
+// CTAs fill the chip on lattices below 2 x 256 sites per SM (16^4: 10.4 against 12.4 us).
 template <typename T, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, sizeof(T) != 4 ? 1 : BLOCK == 256 ? 3 : 5) prolong_kernel(Geom g, const int* __restrict__ sap2dfl, int Ns,
+__global__ void __launch_bounds__(BLOCK, sizeof(T) != 4 ? 1 : BLOCK == 256 ? 3 : 4) prolong_kernel(Geom g, const int* __restrict__ sap2dfl, int Ns,
                                                       const double* b64, const uint4* b16,
                                                       const T* __restrict__ c0, T* psi0, int mode, int nrhs,
                                                       size_t fstride, size_t cstride) {
@@ -492,13 +492,46 @@ __global__ void __launch_bounds__(BLOCK, sizeof(T) != 4 ? 1 : BLOCK == 256 ? 3 :
     load_site_rw<T, 12>(psi, V, i, out);
   }
   const cplx<T>* cc = reinterpret_cast<const cplx<T>*>(c) + (size_t)L * Ns;
-#pragma unroll 4
-  for (int k = 0; k < Ns; ++k) {
+  auto term = [&](int k) {
     cplx<T> ck = cc[k];
     if (mode == 2) ck = -ck;
     load_basis<T>(b64, b16, V, k, i, f);
 #pragma unroll
-    for (int j = 0; j < 12; ++j) out[j] += ck * f[j];      // one rounding per term at the size of the sum
+    for (int j = 0; j < 12; ++j) out[j] += ck * f[j];
+  };
+  if (sizeof(T) == 4 && b16) {
+    if constexpr (sizeof(T) == 4) {
+      // the terms of two basis vectors are summed before they are added to the result: fewer roundings at its size than
+      // one chain, for fewer instructions than a sum per term; the loads of four vectors are in flight together
+      int k = 0;
+#pragma unroll 2
+      for (; k + 1 < Ns; k += 2) {
+        cplx<float> c0 = cc[k], c1 = cc[k + 1];
+        if (mode == 2) { c0 = -c0; c1 = -c1; }
+        uint4 r[2][3];
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+          r[0][u] = __ldg(b16 + ((size_t)k * 3 + u) * V + i);
+          r[1][u] = __ldg(b16 + ((size_t)(k + 1) * 3 + u) * V + i);
+        }
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+          cplx<float> f0[4], f1[4];
+          bf16_unpack4(r[0][u], f0);
+          bf16_unpack4(r[1][u], f1);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            cplx<float> t = c0 * f0[j];
+            cmac(t, c1, f1[j]);
+            out[4 * u + j] += t;
+          }
+        }
+      }
+      if (k < Ns) term(k);
+    }
+  } else {
+#pragma unroll (sizeof(T) == 4 ? 1 : 4)
+    for (int k = 0; k < Ns; ++k) term(k);
   }
   store_site<T, 12>(psi, V, i, out);
   }
