@@ -94,7 +94,8 @@ int dw_create(const dw_params* p, const double* links_host, dw_ctx** out);
 void dw_destroy(dw_ctx* ctx);
 
 /* Free the workspaces a context keeps between calls (solver Krylov fields, the double-float copies
- * of links and clover term); later calls allocate them again.  Synchronises the device. */
+ * of links and clover term, the workspace of ptnet_loss_grad, at most 8 GB, and the scratch pool of
+ * dw_apply with DW_F64X); later calls allocate them again.  Synchronises the device. */
 int dw_release_workspace(dw_ctx* ctx);
 
 /* Bytes of one packed field of precision prec (DW_F64 or DW_F32). */

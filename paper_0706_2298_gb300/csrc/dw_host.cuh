@@ -21,3 +21,14 @@ class DeviceOnce {
     return r;
   }
 };
+
+// alloc(n) for a group of n items, and where memory for so many is not to be had (`short_of`) for half as many, down to
+// one; n is the size it succeeded with, or that of another failure.
+template <typename R, typename F>
+R fit_group(int& n, R short_of, F&& alloc) {
+  for (;;) {
+    const R r = alloc(n);
+    if (r != short_of || n <= 1) return r;
+    n = (n + 1) / 2;
+  }
+}

@@ -402,7 +402,8 @@ cudaError_t launch_dw(dw_ctx* c, const float* local, const float* moved, float2*
   dw_note_launch();
   return cudaGetLastError();
 }
-// fields worked on together: enough for a full GPU, at most 2^19 sites (about 3.7 GB of training workspace)
+// fields worked on together: enough for a full GPU, at most 2^19 sites (about 3.7 GB of training workspace); fewer
+// where the memory is taken
 int pt_group(const dw_ctx* c, int nf) {
   return (int)std::min<long long>(nf, std::max<long long>(1, (1LL << 19) / c->V));
 }
@@ -696,10 +697,14 @@ extern "C" int ptnet_forward(dw_ctx* c, int C, const void* W, int nf, const void
     return DW_EINVAL;
   }
   const size_t fs = (size_t)c->V * 24;
-  const int ng = pt_group(c, nf);
+  int ng = pt_group(c, nf);
   float* acts = nullptr;
-  DW_CUDA(cudaMalloc(&acts, 2 * C * fs * ng * sizeof(float)));
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = fit_group(ng, cudaErrorMemoryAllocation, [&](int n) {
+    const cudaError_t m = cudaMalloc(&acts, 2 * C * fs * n * sizeof(float));
+    if (m != cudaSuccess) cudaGetLastError();
+    return m;
+  });
+  if (e != cudaSuccess) return dw_cuda_fail(e, "ptnet_forward");
   for (int f = 0; f < nf && e == cudaSuccess; f += ng) {
     const int n = std::min(ng, nf - f);
     e = ptnet_forward_impl(c, (const float2*)W, (const float*)x + f * fs, (float*)y + f * fs, acts,
@@ -766,20 +771,28 @@ extern "C" int ptnet_loss_grad(dw_ctx* c, int C, const void* Wv, int nf, const v
   const float2* W = (const float2*)Wv;
   const size_t fs = (size_t)c->V * 24, n = (size_t)c->V * 12;
   const size_t w1 = 9 * 16 * C, w2 = 9 * 16 * C * C, w3 = 9 * 16 * C, nw = w1 + w2 + w3;
-  const int ng = pt_group(c, nf);
-  const size_t np = (size_t)std::max(pt_chunks(c, c->V / PT_S * ng, 9) * 9 * 4096,
-                                     pt_chunks(c, c->V / PT_S * ng, 1) * 9 * 256);
+  int ng = pt_group(c, nf);
   // the workspace stays in the context up to 8 GB: h1, h2, g2, g1 (16 fields each), the output, the gradients
   WsArena& ar = c->ws_solve[4];
-  ar.rewind();
+  float *ws = nullptr, *gw = nullptr;
+  const cudaError_t em = fit_group(ng, cudaErrorMemoryAllocation, [&](int n) {
+    const size_t np = (size_t)std::max(pt_chunks(c, c->V / PT_S * n, 9) * 9 * 4096,
+                                       pt_chunks(c, c->V / PT_S * n, 1) * 9 * 256);
+    ar.rewind();
+    cudaError_t m = ar.get((4 * C + 1) * fs * n * sizeof(float), (void**)&ws);
+    if (m == cudaSuccess) m = ar.get((np + 2 * nw) * sizeof(float2), (void**)&gw);
+    if (m != cudaSuccess) {
+      ar.release();
+      cudaGetLastError();
+    }
+    return m;
+  });
+  if (em != cudaSuccess) return dw_cuda_fail(em, "ptnet_loss_grad");
   struct Keep {
     WsArena& a;
     bool keep;
     ~Keep() { if (!keep) a.release(); }
   } guard{ar, (4 * C + 1) * fs * ng * sizeof(float) <= (size_t)8 << 30};
-  float *ws = nullptr, *gw = nullptr;
-  DW_CUDA(ar.get((4 * C + 1) * fs * ng * sizeof(float), (void**)&ws));
-  DW_CUDA(ar.get((np + 2 * nw) * sizeof(float2), (void**)&gw));
   float* h1 = ws;
   float* h2 = h1 + (size_t)C * fs * ng;
   float* g2 = h2 + (size_t)C * fs * ng;

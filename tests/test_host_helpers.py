@@ -47,6 +47,27 @@ def test_once_per_device(tmp_path):
     """)
 
 
+def test_group_fits_the_memory(tmp_path):
+    """A group that memory cannot be had for is halved down to one; other failures and success end the search."""
+    run(tmp_path, """
+      std::vector<int> tried;
+      int room = 0, n = 0;
+      auto alloc = [&](int k) { tried.push_back(k); return k <= room ? 0 : 2; };
+      n = 8; room = 8;
+      CHECK(fit_group(n, 2, alloc) == 0 && n == 8 && tried == std::vector<int>({8}));
+      tried.clear(); n = 8; room = 3;
+      CHECK(fit_group(n, 2, alloc) == 0 && n == 2 && tried == std::vector<int>({8, 4, 2}));
+      tried.clear(); n = 7; room = 1;
+      CHECK(fit_group(n, 2, alloc) == 0 && n == 1 && tried == std::vector<int>({7, 4, 2, 1}));
+      tried.clear(); n = 5; room = 0;
+      CHECK(fit_group(n, 2, alloc) == 2 && n == 1 && tried == std::vector<int>({5, 3, 2, 1}));
+      tried.clear(); n = 1; room = 0;
+      CHECK(fit_group(n, 2, alloc) == 2 && tried == std::vector<int>({1}));
+      tried.clear(); n = 6;
+      CHECK(fit_group(n, 2, [&](int k) { tried.push_back(k); return 77; }) == 77 && tried == std::vector<int>({6}));
+    """)
+
+
 def test_kernel_limits_go_through_it():
     """No launch keeps the state of its kernel's shared-memory limit for the process as a whole."""
     for name in ("dw_ptnet.cu", "dw_sap.cu"):
