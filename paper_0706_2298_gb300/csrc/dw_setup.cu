@@ -486,9 +486,14 @@ extern "C" int dw_create(const dw_params* p, const double* links_host, dw_ctx** 
     return rc;
   }
   // FP64 links: rows 0 and 1 of a direction, then its row 2
-  for (int mu = 0; mu < 4; ++mu)
-    cudaMemcpy((double*)c->links[DW_F64] + (size_t)mu * 18 * V, l64.data() + (size_t)mu * 12 * V * 8,
-               (size_t)12 * V * 8, cudaMemcpyHostToDevice);
+  for (int mu = 0; mu < 4; ++mu) {
+    const cudaError_t e = cudaMemcpy((double*)c->links[DW_F64] + (size_t)mu * 18 * V,
+                                     l64.data() + (size_t)mu * 12 * V * 8, (size_t)12 * V * 8, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      free_ctx(c);
+      return dw_cuda_fail(e, "cudaMemcpy");
+    }
+  }
   link_row2_kernel<<<(unsigned)((4 * V + 255) / 256), 256>>>(V, (double2*)c->links[DW_F64]); dw_note_launch();
   cudaMemset(c->d_count, 0, 64 * sizeof(unsigned));
   if (cudaMallocHost((void**)&c->h_red, 1 << 16) != cudaSuccess) {
