@@ -2,6 +2,9 @@
 // Reductions accumulate in FP64 with a fixed order: per-thread partial
 // sums, warp shuffles, one partial per CTA, and the last CTA to finish adds
 // the CTA partials in index order -> results are deterministic.
+#include <algorithm>
+#include <mutex>
+
 #include "dw_common.cuh"
 
 namespace {
@@ -546,16 +549,26 @@ int dw_make_dd(dw_ctx* c, cudaStream_t s) {
 }
 
 cudaError_t dw_pool_alloc(dw_ctx* c, size_t bytes, void** p, cudaStream_t s) {
-  if (!c->pool) {
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = c->device;
-    cudaError_t e = cudaMemPoolCreate(&c->pool, &props);
-    if (e != cudaSuccess) return e;
-    uint64_t keep = std::max<uint64_t>((uint64_t)4 * c->V * 24 * sizeof(double), 64u << 20);   // a pool grows by 32 MB
-    e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    if (e != cudaSuccess) return e;
+  static std::mutex making;              // two threads may make their first call at once
+  cudaMemPool_t pool;
+  {
+    std::lock_guard<std::mutex> hold(making);
+    if (!c->pool) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = c->device;
+      cudaError_t e = cudaMemPoolCreate(&pool, &props);
+      if (e != cudaSuccess) return e;
+      uint64_t keep = std::max<uint64_t>((uint64_t)4 * c->V * 24 * sizeof(double), 64u << 20);   // a pool grows by 32 MB
+      e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+      if (e != cudaSuccess) {
+        cudaMemPoolDestroy(pool);
+        return e;
+      }
+      c->pool = pool;
+    }
+    pool = c->pool;
   }
-  return cudaMallocFromPoolAsync(p, bytes, c->pool, s);
+  return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
