@@ -280,8 +280,8 @@ int gcr_solve(dw_ctx* ctx, dfl_ctx* d, const sol_params* p, int nrhs, const doub
 int dw_autotune(dw_ctx* ctx, int nrhs, char* report, size_t report_len);
 
 /* Shape sweep of the FP32 cooperative little solver of d: grid sizes (all SMs, 3/4 and 1/2 of them)
- * x kernel (the one compiled for Ns with one reduction per step, "ring" in the summary / the generic
- * one), timed with CUDA events on little solves of a fixed right-hand side; the fastest per
+ * x kernel (the one compiled for Ns, called "ring" in the summary, / the generic one, "registers"),
+ * timed with CUDA events on little solves of a fixed right-hand side; the fastest per
  * iteration is kept in d.  JSON summary in report (may be NULL).  Synchronous. */
 int dfl_autotune(dfl_ctx* d, char* report, size_t report_len);
 

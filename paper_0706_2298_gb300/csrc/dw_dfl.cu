@@ -1193,25 +1193,26 @@ DW_D void coop_row_range(int nrow, int* rb, int* re) {
   *re = min(nrow, *rb + R);
 }
 
-// y = B^ x = x - M_eo (M_oe x); ends with a grid barrier.  The CTA barriers on both sides of
-// the grid barriers are redundant for correctness but halve the solver's run time on GB300
-// (measured: 3.8 ms -> 1.9 ms for 42 iterations at Nb = 2592, Ns = 20).
+// the hop to the rows of one parity
 template <typename T, int NS>
-DW_D void hop_any(const CoopArgs<T>& a, bool odd, const cplx<T>* src, const cplx<T>* corr, cplx<T> cs,
+DW_D void coop_hop_to(const CoopArgs<T>& a, bool odd, const cplx<T>* src, const cplx<T>* corr, cplx<T> cs,
                   const cplx<T>* base, cplx<T>* out, T sign, cplx<T>* hp) {
   coop_hop<T, NS>(odd ? a.No : a.Ne, a.Ns, odd ? a.list_o : a.list_e, odd ? a.lnb_o : a.lnb_e, a.M, src, corr, cs, base,
                   out, sign, hp);
 }
 
+// y = B^ x = x - M_eo (M_oe x); ends with a grid barrier.  The CTA barriers on both sides of
+// the grid barriers are redundant for correctness but halve the solver's run time on GB300
+// (measured: 3.8 ms -> 1.9 ms for 42 iterations at Nb = 2592, Ns = 20).
 template <typename T, int NS>
 DW_D void coop_bhat(cg::grid_group& grid, const CoopArgs<T>& a, const cplx<T>* x, cplx<T>* tmpo, cplx<T>* y,
                     cplx<T>* hp) {
   const cplx<T> zero = {T(0), T(0)};
-  hop_any<T, NS>(a, true, x, nullptr, zero, nullptr, tmpo, T(1), hp);     // tmpo = M_oe x
+  coop_hop_to<T, NS>(a, true, x, nullptr, zero, nullptr, tmpo, T(1), hp);     // tmpo = M_oe x
   __syncthreads();
   grid.sync();
   __syncthreads();
-  hop_any<T, NS>(a, false, tmpo, nullptr, zero, x, y, T(-1), hp);         // y = x - M_eo tmpo
+  coop_hop_to<T, NS>(a, false, tmpo, nullptr, zero, x, y, T(-1), hp);         // y = x - M_eo tmpo
   __syncthreads();
   grid.sync();
   __syncthreads();
@@ -1356,12 +1357,12 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) little_gcr_coop_kernel(CoopAr
       // this CTA's own rows, so no grid barrier follows it
       slice([&](size_t i) { xk[i] = rk[i]; });
       const cplx<T> acs = k > 0 ? cplx<T>{sh.ac[0], sh.ac[1]} : zero;
-      hop_any<T, NS>(a, true, k > 0 ? rhob[cur ^ 1] : rk, k > 0 ? chi(k - 1) : nullptr, acs, nullptr, tmpo,
-                           T(1), hp);
+      coop_hop_to<T, NS>(a, true, k > 0 ? rhob[cur ^ 1] : rk, k > 0 ? chi(k - 1) : nullptr, acs, nullptr, tmpo,
+                         T(1), hp);
       __syncthreads();
       grid.sync();
       __syncthreads();
-      hop_any<T, NS>(a, false, tmpo, nullptr, zero, rk, ck, T(-1), hp);
+      coop_hop_to<T, NS>(a, false, tmpo, nullptr, zero, rk, ck, T(-1), hp);
       // one reduction: u = g^+ chi_k (A.3), the raw coefficients (chi'_j, chi_k), j < k, and |rho_k|^2
       if (a.a3) cta_dots<T>(sh, gV, vn, ns, ck, sl, 0);
       if (k > 0) cta_dots<T>(sh, chiV, vn, k, ck, sl, na);
