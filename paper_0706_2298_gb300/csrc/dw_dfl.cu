@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(128 * RK_G, sizeof(T) == 4 ? 2 : 1) restrict_n
 // (the groups of a batch are neighbouring CTAs), so a basis value is read and unpacked once per RT of them.  One unit
 // of the basis (four components) at a time: RT x 4 field components, 4 basis components and 2 RT Ns / RK_G sums
 // stay within the 128 registers of 512 threads.  Bound: issue and the latency of the loads (16 warps per SM).  12 fields
-// of 24x16^3, Ns = 20: 100 us.
+// of 24x16^3, Ns = 20: 101 us.
 template <int NS, int RT>
 __global__ void __launch_bounds__(128 * RK_G, 1) restrict_batch_kernel(Geom g, const int* __restrict__ sub, int nsub,
                                                                         const uint4* __restrict__ b16,
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(BLOCK, sizeof(T) != 4 ? 1 : BLOCK == 256 ? 3 :
 
 // psi_r = Phi c_r for batches with the BF16 basis: a thread holds one site of RT right-hand sides (24 RT
 // accumulators), so a basis value is read and unpacked once per RT of them; the groups of a batch are neighbouring CTAs.  Bound: issue
-// (12 warps per SM).  12 fields of 24x16^3, Ns = 20: 81 us; this and the restriction
+// (12 warps per SM).  12 fields of 24x16^3, Ns = 20: 90 us (81 as one chain, further from FP64); this and the restriction
 // together took 377 us with one field after the other in a CTA and the basis from L2.
 template <int RT>
 __global__ void __launch_bounds__(128, 3) prolong_batch_kernel(Geom g, const int* __restrict__ sap2dfl, int Ns,
@@ -558,8 +558,8 @@ __global__ void __launch_bounds__(128, 3) prolong_batch_kernel(Geom g, const int
   for (int r = 0; r < RT; ++r)
 #pragma unroll
     for (int j = 0; j < 12; ++j) out[r][j] = {0.f, 0.f};
-  // two basis vectors at a time, their terms summed before they are added to the result: fewer roundings at its size than
-  // one chain, for fewer instructions than a sum per term; the last one of an odd Ns by itself
+  // four basis vectors at a time, their terms summed before they are added to the result: fewer roundings at its size than
+  // one chain, for an eighth more instructions; the remaining ones of an Ns that four does not divide one by one
   auto add = [&](int k, auto nk) {
     constexpr int NK = decltype(nk)::value;
     cplx<float> ck[NK][RT];
@@ -580,15 +580,17 @@ __global__ void __launch_bounds__(128, 3) prolong_batch_kernel(Geom g, const int
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           cplx<float> s = ck[0][r] * f[0][j];
-          if (NK > 1) cmac(s, ck[NK - 1][r], f[NK - 1][j]);
+#pragma unroll
+          for (int q = 1; q < NK; ++q) cmac(s, ck[q][r], f[q][j]);
           out[r][4 * u + j] += s;
         }
     }
   };
   int k = 0;
 #pragma unroll 1
-  for (; k + 1 < Ns; k += 2) add(k, std::integral_constant<int, 2>());
-  if (k < Ns) add(k, std::integral_constant<int, 1>());
+  for (; k + 3 < Ns; k += 4) add(k, std::integral_constant<int, 4>());
+#pragma unroll 1
+  for (; k < Ns; ++k) add(k, std::integral_constant<int, 1>());
 #pragma unroll
   for (int r = 0; r < RT; ++r)
     if (r < nr) store_site<float, 12>(psi0 + (size_t)(r0 + r) * fstride, V, i, out[r]);

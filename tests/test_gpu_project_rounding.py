@@ -78,9 +78,9 @@ def test_error_against_plain_single_precision(L, bs, Ns):
     assert rel(got, want) <= BOUND * rel(prolongation(phi, z, np.float32), want)
 
 
-@pytest.mark.parametrize("Ns,nrhs", [(5, 2), (5, 6), (13, 3)])
-def test_batch_with_an_odd_subspace(Ns, nrhs, monkeypatch):
-    """The batched prolongation takes two basis vectors at a time: the last one of an odd number by itself.  (Without it
+@pytest.mark.parametrize("Ns,nrhs", [(3, 2), (5, 2), (5, 6), (6, 4), (7, 5), (13, 3)])
+def test_batch_with_remaining_vectors(Ns, nrhs, monkeypatch):
+    """The batched prolongation takes four basis vectors at a time, those that remain one by one.  (Without them
     the coarse corrections miss a mode and the solver does not reach 1e-10 in a similar number of steps.)"""
     L = (8, 8, 8, 8)
     ctx = dw.dw_create(L, -0.1, 1.0, synth.random_gauge(L, 75), (4, 4, 4, 4))
