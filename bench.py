@@ -62,9 +62,9 @@ PLAIN_COUNTS = os.path.join(ROOT, "paper_0706_2298_gb300", "plain_gcr_counts.jso
 
 # DRAM bytes per little-GCR iteration of the cooperative kernel, from one ncu capture of the
 # current kernel (dram__bytes_read.sum + dram__bytes_write.sum of one launch / its iterations):
-# 48x24^3, Ns = 20: (75.18 + 3.30) MB over 41 iterations (cold cache: the first iteration reads
+# 48x24^3, Ns = 20: (75.22 + 3.20) MB over 43 iterations (cold cache: the first iteration reads
 # the little operator from HBM, the rest hit L2).  Remove an entry when the kernel changes.
-LITTLE_TRAFFIC = {("24^3x48", 20): 78.48e6 / 41}
+LITTLE_TRAFFIC = {("24^3x48", 20): 78.42e6 / 43}
 
 
 def aggregate_ranks(t_ms, steps, world, device="cpu"):
